@@ -5,42 +5,53 @@
 // Persistent kernel, one CTA per SM; CTA k takes instances k, k + grid, ...
 // An instance's queries stream through a ring of shared-memory stages in
 // tiles of up to 128 (TMA, 128-byte swizzle) and are read from HBM once.
+// Both contractions of a tile run on the tensor cores (tcgen05):
 //
-// Screening on the tensor cores: per tile, D1 = Q x [c_hi ; c_lo]^T where
-// c_hi = bf16(c / |c|) and c_lo = bf16(c / |c| - c_hi), so dot_b = D1[:, b] +
-// D1[:, nbp + b] carries the unit-centroid dot to about 2^-16 |q| (bf16 x bf16
-// products are exact, the accumulation is fp32); D2 = Q x Q^T gives |q|^2 on
-// its diagonal.  When best and second-best dots differ by at most 1e-4 |q|
-// (about twice the bound on their difference's error: 2^-17 |q| per dot from
-// the hi/lo split, 128 fp32 accumulation steps), the query is re-decided
-// exactly: the beacon maximising (q . c_b) / |c_b| in double-float arithmetic
-// (exact products, TwoSum accumulation, 1 / |c_b| from a double-float sum of
-// squares and one Newton step, to about 2^-44 relative), which
-// agrees with the cosine (q . c_b) / (|q| |c_b|) evaluated in fp64 except at
-// ties below ~1e-12 (the lowest beacon wins ties).  Zero queries and instances
-// without a valid beacon give -1.
+// Screening: D1 = Q x [c_hi ; c_lo]^T where c_hi = bf16(c / |c|) and c_lo =
+// bf16(c / |c| - c_hi), so dot_b = D1[:, b] + D1[:, nbp + b] carries the
+// unit-centroid dot to about 2^-16 |q| (bf16 x bf16 products are exact, the
+// accumulation is fp32).  When best and second-best dots differ by at most
+// 1e-4 |q| (about twice the bound on their difference's error: 2^-17 |q| per
+// dot from the hi/lo split, 128 fp32 accumulation steps; |q| is taken a few
+// percent too large), the query is re-decided exactly: the beacon maximising
+// (q . c_b) / |c_b| in double-float arithmetic (exact products, TwoSum
+// accumulation, 1 / |c_b| from a double-float sum of squares and one Newton
+// step, to about 2^-44 relative), which agrees with the cosine (q . c_b) /
+// (|q| |c_b|) evaluated in fp64 except at ties below ~1e-12 (the lowest beacon
+// wins ties).  Only beacons screened within 2e-4 |q| of the best enter that
+// comparison.  Zero queries and instances without a valid beacon give -1.
 //
-// Sums: int64 fixed point with 40 fractional bits.  A tile's screened rows
-// are sorted by beacon (ballot counting sort); each accumulator warp takes an
-// equal slice of that order, its lanes owning D / 32 columns each, and keeps
-// three fp32 part sums per column that are exact by construction (see Parts;
-// exact for 2^-31 <= |x| < 2^14, the conversion to fixed point per beacon
-// change rather than per element); re-decided rows are converted directly.
-// The per-call sum is exact and independent of the order.  It is then
-// added once to the fp64 running sum, correctly rounded (fold_sum_fp64: one
-// fp64 addition while the call's sum is exact in fp64, fold_sum's exact
-// integer addition beyond; the bookkeeping warps that fold have the fp64 pipe
-// to themselves), and c = fp32(sum / count) to within one fp32 ulp from
+// Sums: Q^T x A, where A is the tile's one-hot assignment matrix (128 queries x
+// beacons), exact: an element x with |x| < 2^E (E chosen per instance) goes
+// whole into one of two operands, the tile itself (|x| >= 2^(E-10), a multiple
+// of 2^(E-17)) or a second tile (smaller ones, multiples of 2^(E-27) for
+// |x| >= 2^(E-20)), whose sums over 128 rows stay below 2^24 grid steps, so the
+// fp32 accumulator never rounds.  The two sums of a (column, beacon) cell become
+// one 64-bit integer per tile, added up in a register per cell.  The few
+// elements outside [2^(E-20), 2^E) (one in ten tiles of normal data) are
+// zeroed in the operands and go to the fold as a list (past 32 per instance
+// through a global array of this CTA).  E comes from the largest |q| this CTA has seen (before that from
+// the centroids), never below -11, so that what the operands hold is exact
+// in fixed point with 40 fractional bits; the result does not depend on it.
+// The call's sum is then added once to the fp64 running sum, correctly rounded
+// (fold_sum, in integers: fp64 is slow on this part), and c = fp32(sum / count) to within one fp32 ulp from
 // double-float arithmetic on the sum's bits.
 //
-// Warp roles (26 warps): warp 0 TMA producer; warp 1 TMEM allocation and MMA
-// issue; warps 2..5 screeners (one per TMEM lane quarter: decisions, the
-// sorted row list of the tile, exact re-decisions); warps 6..21 accumulators
-// (the sums of a tile, while the screeners work on the next one; the row
-// lists are double-buffered); warps 22..25 bookkeeping: they build the
-// unit-centroid operand of the next instance and fold the finished one into
-// the running state, from centroids and sums brought in by bulk copies
-// (accumulators double-buffered by instance).  All waits are bounded.
+// Warp roles (23 warps): warp 0 TMA producer; warp 1 TMEM allocation and the
+// screening MMAs; warp 2 the sums' MMAs; warps 3..10 two groups of four that
+// take alternate tiles, one query per thread (its decision, the split of its
+// elements, its column of A); warps 11..18 one column of d and half of the
+// beacons per thread: they take the sums out of tensor memory and fold them
+// into the running state; warps 19..22 build the unit-centroid operand of the
+// next instances.  All waits are bounded.
+//
+// What bounds it: the roles' instruction streams.  About 9 K warp instructions per
+// tile at 40 % issue, a quarter of the stalls instruction fetch (hence the loops
+// kept small), with two tiles in flight per SM because shared memory holds no
+// third second-tile.  The sums took most of the time when they were formed in fp32
+// parts by CUDA cores from rows sorted by beacon (about 14 K warp instructions
+// per tile): 4608 instances x 512 queries of 128, 8 beacons: 393 us, now 298 (95 at
+// the copy rate); 8192 instances, 16 beacons: 815 us, now 537 (206).
 #include "bkv_device.cuh"
 #include "bkv_internal.h"
 #include "k_update_math.cuh"
@@ -48,15 +59,23 @@
 namespace bkv {
 namespace {
 
-constexpr int kScreeners = 4;
-constexpr int kAccum = 16;
-constexpr int kKeepers = 4;
-constexpr int kUThreads = 32 * (2 + kScreeners + kAccum + kKeepers);
-constexpr int kQTile = 128;                 // queries per tile (MMA M)
+constexpr int kGroups = 2;                  // row groups of four warps, one tile each
+constexpr int kGroupWarp0 = 3;              // first of the row groups' warps
+constexpr int kSumWarp0 = kGroupWarp0 + 4 * kGroups;  // first of the eight warps that take the sums
+constexpr int kBuildWarp0 = kSumWarp0 + 8;
+constexpr int kUThreads = 32 * (kBuildWarp0 + 4);
+constexpr int kQTile = 128;                 // queries per tile (MMA M of the screening, K of the sums)
 constexpr uint32_t kQBox = 128 * 128;       // [128 rows][64 bf16] swizzled box slot
-constexpr int kUMaxStages = 8;
-constexpr size_t kUSmemBudget = 216 * 1024;
-constexpr int kGroup = 4;  // rows an accumulator lane sums per step when they share a beacon
+constexpr int kUMaxStages = 6;
+constexpr int kDots = 3;                    // screening accumulators in tensor memory
+constexpr int kSums = 4;                    // sum accumulators: a fold may take as long as its instance's tiles
+constexpr int kSlots = 16;                  // per-instance words in flight between the roles (at most 11 instances)
+constexpr int kSpillSlots = 8;              // instances whose spilled elements may be in flight
+constexpr int kSpillList = 32;              // spilled elements per instance kept in shared memory
+constexpr size_t kUSmemBudget = 220 * 1024;
+constexpr int kMinE = -11, kMaxE = 14;
+constexpr int kLargeBits = 10;              // octaves below 2^E that the tile itself holds
+constexpr int kSmallBits = 20;              // octaves below 2^E that the operands hold
 
 struct UpdArgs {
   int n_inst, nq, nb, nbp;  // instances, queries per instance, beacons, beacons padded to 8
@@ -65,27 +84,27 @@ struct UpdArgs {
   double* sums;
   long long* counts;
   int* assign_out;
+  unsigned long long* spill;  // [grid][kSpillSlots][nb][D], zero between instances
   int* err;
 };
 
-template <int D>
+// NBO: beacons padded to 16 (the N of the sums' MMA).
+template <int D, int NBO>
 struct UpdCfg {
   static constexpr int kBoxes = D / 64;
   static constexpr uint32_t kStageBytes = kBoxes * kQBox;
-  __host__ __device__ static size_t bmat_bytes(int nbp) { return static_cast<size_t>(kBoxes) * 2 * nbp * 128; }
-  __host__ __device__ static size_t state_bytes(int nb, int nbp) {
-    // bmat[2], acc[2] (int64), cent[2] (fp32), sums (fp64)
-    return 2 * bmat_bytes(nbp) + 2 * static_cast<size_t>(nb) * D * 8 + 2 * static_cast<size_t>(nb) * D * 4 +
-           static_cast<size_t>(nb) * D * 8;
+  static constexpr uint32_t kHotBytes = 2 * NBO * 128;    // one-hot operand: two 64-query boxes of NBO rows
+  static constexpr int kParts = D == 128 ? 2 : 1;         // accumulators per tile (d = 64: both operands in one)
+  static constexpr uint32_t kXchg = D == 64 ? 64 * NBO * 4 : 0;  // d = 64: the small parts' sums at a fold
+  __host__ __device__ static uint32_t bmat_bytes(int nbp) { return static_cast<uint32_t>(kBoxes) * 2 * nbp * 128; }
+  __host__ __device__ static uint32_t fixed_bytes(int nbp) {
+    return kGroups * (kStageBytes + kHotBytes) + 2 * bmat_bytes(nbp) + kXchg;
   }
-  static int stages(int nb, int nbp) {
-    const size_t room = kUSmemBudget - 1024 - state_bytes(nb, nbp);
-    const int n = static_cast<int>(room / kStageBytes);
+  static int stages(int nbp) {
+    const int n = static_cast<int>((kUSmemBudget - 1024 - fixed_bytes(nbp)) / kStageBytes);
     return n < kUMaxStages ? n : kUMaxStages;
   }
-  static size_t smem_bytes(int nb, int nbp) {
-    return 1024 + static_cast<size_t>(stages(nb, nbp)) * kStageBytes + state_bytes(nb, nbp);
-  }
+  static size_t smem_bytes(int nbp) { return 1024 + static_cast<size_t>(stages(nbp)) * kStageBytes + fixed_bytes(nbp); }
 };
 
 __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity, int* err) {
@@ -95,12 +114,9 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity, int* 
 
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// Contiguous global -> shared copy by the TMA unit, completing on `bar`.
-__device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
+// Brings `bytes` (a multiple of 16) at p into L2.
+__device__ __forceinline__ void bulk_prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(p)), "r"(bytes) : "memory");
 }
 
 // round(x * 2^40) of the bf16 value whose bits sit in the upper half of
@@ -117,543 +133,786 @@ __device__ __forceinline__ uint32_t sw128_offset(int row, int col, uint32_t box_
   return (col >> 6) * box_bytes + row * 128 + ((((col & 63) >> 3) ^ (row & 7)) << 4) + ((col & 7) << 1);
 }
 
-// Adds the kCols bf16 values at p (columns col0 ..) to s as fixed point.
-template <int kCols>
-__device__ __forceinline__ void add_fixed(long long (&s)[kCols], const unsigned char* p) {
-  if constexpr (kCols == 4) {
-    const uint2 w = *reinterpret_cast<const uint2*>(p);
-    s[0] += bf16_fixed40(w.x << 16);
-    s[1] += bf16_fixed40(w.x & 0xffff0000u);
-    s[2] += bf16_fixed40(w.y << 16);
-    s[3] += bf16_fixed40(w.y & 0xffff0000u);
-  } else {
-    const uint32_t w = *reinterpret_cast<const uint32_t*>(p);
-    s[0] += bf16_fixed40(w << 16);
-    s[1] += bf16_fixed40(w & 0xffff0000u);
+// Shared-memory descriptor of an operand read across its rows (MN-major): 64 elements of a row per
+// 128-byte line, 8-row groups 1024 B apart, the next 64 elements `lbo` bytes further; 128-byte swizzle.
+__device__ __forceinline__ uint64_t sdesc_mnmajor_sw128(uint32_t smem_addr, uint32_t lbo) {
+  return (sdesc_kmajor_sw128(smem_addr) & ~(0x3FFFull << 16)) | (static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16);
+}
+
+// 16-byte shared-memory store where cond is not 0, predicated rather than branched around.
+__device__ __forceinline__ void st_shared_v4_if(uint32_t cond, void* p, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.u32 p, %0, 0;\n\t"
+      "@p st.shared.v4.b32 [%1], {%2, %3, %4, %5};\n\t}" ::"r"(cond),
+      "r"(smem_u32(p)), "r"(x), "r"(y), "r"(z), "r"(w)
+      : "memory");
+}
+
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// bf16 bits of 2^k, in both halves of a word.
+__device__ __forceinline__ uint32_t pow2_bf16x2(int k) {
+  const uint32_t b = static_cast<uint32_t>(k + 127) << 7;
+  return b | (b << 16);
+}
+
+__device__ __forceinline__ __nv_bfloat162 as_bf162(uint32_t w) { return *reinterpret_cast<__nv_bfloat162*>(&w); }
+
+// 8 consecutive fp32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Exact assignment of query n of the tile (its elements are in `raw` or, where that holds 0, in `small`)
+// among the candidate beacons (warp-wide): the valid beacon
+// maximising (q . c_b) * (1 / |c_b|) in double-float arithmetic, ties to the lower beacon, -1 for a zero
+// query (exact_decision's result: the same operations, with a candidate's dot and norm formed together
+// and the next candidate's row already loading).  Out of line: rare.
+template <int D>
+__device__ __noinline__ int refine_row(const unsigned char* raw, const unsigned char* small, int n, const float* cent_e,
+                                       uint32_t cand) {
+  const int lane = threadIdx.x & 31;
+  float x[D / 32], c[D / 32];
+  int b = __ffs(cand) - 1;
+#pragma unroll
+  for (int j = 0; j < D / 32; ++j) {
+    const uint32_t off = sw128_offset(n, lane + 32 * j, kQBox);
+    const uint32_t w = *reinterpret_cast<const uint16_t*>(raw + off) | *reinterpret_cast<const uint16_t*>(small + off);
+    x[j] = __uint_as_float(w << 16);
+    c[j] = cand ? cent_e[b * D + lane + 32 * j] : 0.f;
   }
+  int nz = 0;
+#pragma unroll
+  for (int j = 0; j < D / 32; ++j) nz |= x[j] != 0.f;
+  if (!__any_sync(0xffffffffu, nz)) return -1;
+  DF best{-INFINITY, 0.f};
+  int best_b = -1;
+  while (cand) {
+    cand &= cand - 1;
+    const int b_next = __ffs(cand) - 1;
+    float c_next[D / 32];
+#pragma unroll
+    for (int j = 0; j < D / 32; ++j) c_next[j] = cand ? cent_e[b_next * D + lane + 32 * j] : 0.f;
+    float n2 = 0.f;
+    DF n2d{0.f, 0.f}, dt{0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < D / 32; ++j) {
+      n2 = fmaf(c[j], c[j], n2);
+      n2d = df_add(n2d, df_two_prod(c[j], c[j]));
+      dt = df_add(dt, df_two_prod(x[j], c[j]));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+      n2d = df_add(n2d, DF{__shfl_xor_sync(0xffffffffu, n2d.hi, o), __shfl_xor_sync(0xffffffffu, n2d.lo, o)});
+      dt = df_add(dt, DF{__shfl_xor_sync(0xffffffffu, dt.hi, o), __shfl_xor_sync(0xffffffffu, dt.lo, o)});
+    }
+    bool plain = true;
+    const DF cs = df_mul(dt, centroid_inv_norm(n2d, n2, plain));
+    if (best_b < 0 || df_gt(cs, best)) {
+      best = cs;
+      best_b = b;
+    }
+    b = b_next;
+#pragma unroll
+    for (int j = 0; j < D / 32; ++j) c[j] = c_next[j];
+  }
+  return best_b;
 }
 
-// *cell += v on a shared int64 cell, as two 32-bit atomic additions: the low word's carry-out is
-// decided by the value that addition found, so concurrent additions still sum exactly (a 64-bit
-// shared-memory atomic addition is a compare-and-swap loop on this part).
-__device__ __forceinline__ void shared_add_i64(long long* cell, long long v) {
-  uint32_t* w = reinterpret_cast<uint32_t*>(cell);
-  const uint32_t lo = static_cast<uint32_t>(v);
-  const uint32_t old = atomicAdd(w, lo);
-  const uint32_t carry = old + lo < old ? 1u : 0u;
-  const uint32_t hi = static_cast<uint32_t>(static_cast<unsigned long long>(v) >> 32) + carry;
-  if (hi != 0u) atomicAdd(w + 1, hi);
+// cnt[b] += the number of lanes whose mine == b (mine < 0: none), for every b < NB: five 6-bit counters per
+// warp sum, then one conflict-free addition per beacon (one atomic per lane would serialise).
+template <int NB>
+__device__ __forceinline__ void add_counts(int* cnt, int mine) {
+  const int lane = threadIdx.x & 31;
+  constexpr int kWords = (NB + 4) / 5;
+  uint32_t tot = 0u;
+#pragma unroll
+  for (int w = 0; w < kWords; ++w) {
+    const int k = mine - 5 * w;
+    const uint32_t sum = __reduce_add_sync(0xffffffffu, k >= 0 && k < 5 ? 1u << (6 * k) : 0u);
+    tot = lane / 5 == w ? sum : tot;
+  }
+  const int n = static_cast<int>((tot >> (6 * (lane % 5))) & 63u);
+  if (lane < NB && n > 0) atomicAdd(&cnt[lane], n);
 }
 
-// The same split for two adjacent columns at once, on packed f32x2 values
-// (low word: the first column), with Blackwell's paired fp32 adds.
-struct Parts2 {
-  unsigned long long h, m, l;
+// Spilled elements of one instance: the first kSpillList as (beacon << 8 | column, fixed point) here, more
+// in the CTA's global array.
+struct SpillList {
+  int n;
+  int key[kSpillList];
+  long long val[kSpillList];
 };
 
-__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
-// w holds two bf16 values (low half: the first column).
-__device__ __forceinline__ void parts2_add(Parts2& p, uint32_t w) {
-  constexpr unsigned long long kM1 = 0x49C0000049C00000ull;  // {1.5 * 2^20, 1.5 * 2^20}
-  constexpr unsigned long long kM2 = 0x4140000041400000ull;  // {12, 12}
-  const unsigned long long x = static_cast<unsigned long long>(w << 16) |
-                               (static_cast<unsigned long long>(w & 0xffff0000u) << 32);
-  const unsigned long long xh = f2_sub(f2_add(x, kM1), kM1);
-  const unsigned long long r = f2_sub(x, xh);
-  const unsigned long long xm = f2_sub(f2_add(r, kM2), kM2);
-  p.h = f2_add(p.h, xh);
-  p.m = f2_add(p.m, xm);
-  p.l = f2_add(p.l, f2_sub(r, xm));
-}
-
-// Column `second` (0 or 1) of a packed pair of part sums.
-__device__ __forceinline__ Parts parts2_get(const Parts2& p, int second) {
-  const int sh = second ? 32 : 0;
-  return Parts{__uint_as_float(static_cast<uint32_t>(p.h >> sh)), __uint_as_float(static_cast<uint32_t>(p.m >> sh)),
-               __uint_as_float(static_cast<uint32_t>(p.l >> sh))};
-}
-
+// The elements of one row (n of the tile) that the operands cannot hold: |x| >= 2^E (or not finite), which
+// sit in the tile, and 0 < |x| < 2^(E - 20), which sit in the second one.  Each is zeroed there and noted
+// for the row's beacon (b < 0: the row is not assigned).  Warp-wide; returns whether some went to the
+// global array.  Out of line: rare.
 template <int D>
+__device__ __noinline__ bool spill_row(unsigned char* raw, unsigned char* small, int n, int E, int b, SpillList* list,
+                                       unsigned long long* spill) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t hi = pow2_bf16x2(E) & 0xffffu, lo = pow2_bf16x2(E - kSmallBits) & 0xffffu;
+  constexpr int kC = D / 32;  // this lane's columns
+  bool over = false;
+#pragma unroll
+  for (int k = 0; k < kC; ++k) {
+    const int col = lane * kC + k;
+    const uint32_t off = sw128_offset(n, col, kQBox);
+    uint16_t* in_raw = reinterpret_cast<uint16_t*>(raw + off);
+    uint16_t* in_small = reinterpret_cast<uint16_t*>(small + off);
+    const uint32_t w = *in_raw | *in_small, m = w & 0x7fffu;  // one of the two is zero
+    if (m == 0u || (m >= lo && m < hi)) continue;
+    *in_raw = 0;
+    *in_small = 0;
+    if (b < 0) continue;
+    const float x = __uint_as_float(w << 16);
+    const long long f = fabsf(x) < 16384.f ? fixed40_one(x) : bf16_fixed40(w << 16);
+    const int at = atomicAdd(&list->n, 1);
+    if (at < kSpillList) {
+      list->key[at] = (b << 8) | col;
+      list->val[at] = f;
+    } else {
+      atomicAdd(spill + b * D + col, static_cast<unsigned long long>(f));
+      over = true;
+    }
+  }
+  if (!__any_sync(0xffffffffu, over)) return false;
+  __threadfence();
+  return true;
+}
+
+template <int D, int NBO>
 __global__ void __launch_bounds__(kUThreads, 1)
     update_kernel(const __grid_constant__ CUtensorMap qmap, UpdArgs a, int n_stages) {
-  using C = UpdCfg<D>;
-  constexpr int kCols = D / 32;  // columns per lane in the accumulation
+  using C = UpdCfg<D, NBO>;
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[kUMaxStages], empty_bar[kUMaxStages];
-  __shared__ __align__(8) uint64_t accfull[2], accfree[2], bready[2], bfree[2], drain_bar;
-  __shared__ __align__(8) uint64_t accdone[2], accclear[2], cbar[2], sbar, sfull[2], sempty[2];
+  __shared__ __align__(8) uint64_t accfull[kDots], accfree[kDots], bready[2], bfree[2], drain_bar[2];
+  __shared__ __align__(8) uint64_t sumready[kGroups], smallfree[kGroups], sumfull[kSums], cntready[kSums], sumfree[kSums];
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
-  __shared__ int order_t[2][kQTile];  // row | beacon << 8, sorted by beacon (by tile parity)
-  __shared__ int refine_t[2][kQTile];
-  __shared__ int n_refine[2], n_asg_sh[2];
-  __shared__ int cnt_w[2][4][kMaxBeacons];
-  __shared__ int add_cnt[2][kMaxBeacons];
-  __shared__ int bvalid[2][kMaxBeacons];
-  __shared__ DF cninv[2][kMaxBeacons];  // 1 / |c_b| as a double-float
-  __shared__ long long cnt_old[2][kMaxBeacons];
-  __shared__ DF rcp_sh[kMaxBeacons];  // 1 / count after this call, as a double-float
-  __shared__ int degenerate[2];
+  __shared__ uint32_t seen_sh;               // largest |q|^2 below 2^(2 kMaxE) seen so far (fp32 bits)
+  // per instance in flight
+  __shared__ uint32_t vmask_sh[kSlots];      // valid beacons (count > 0, nonzero centroid)
+  __shared__ int exp_sh[kSlots];             // E; bit 8: a centroid norm is extreme, every query is re-decided
+  __shared__ int add_cnt[kSlots][kMaxBeacons];  // queries assigned so far
+  __shared__ int spilled_sh[kSlots];         // elements or sums went to the global array
+  __shared__ SpillList list_sh[kSpillSlots];
+  __shared__ uint32_t kv_sh[4];              // builders: each warp's valid beacons
+  __shared__ uint32_t km_sh[4];              // builders: each warp's largest |c|^2 (fp32 bits), bit 31: extreme norm
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nq = a.nq, nb = a.nb, nbp = a.nbp;
-  const int cells = nb * D;
   const int n_my = blockIdx.x < a.n_inst ? (a.n_inst - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
   const int T = (nq + kQTile - 1) / kQTile;  // tiles per instance
+  const int n_tiles = n_my * T;
   const int ncols1 = 2 * nbp;                 // screening columns (hi, lo)
-  const int acc_cols = ncols1 + kQTile;       // + the Q Q^T block
   const uint32_t bbox = static_cast<uint32_t>(ncols1) * 128;  // bytes of one 64-column box of bmat
 
   // 1024-byte aligned (the 128-byte swizzle pattern repeats every 1024 bytes);
   // offset from the __shared__ array itself so that accesses stay shared-space
   unsigned char* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  unsigned char* stage_smem = base;                                             // [n_stages][kBoxes][128 x 128 B]
-  unsigned char* bmat = base + static_cast<size_t>(n_stages) * C::kStageBytes;  // [2][kBoxes][2 nbp x 128 B]
-  // [2][nb][D]; column 4 l + c of a beacon row (l = lane, c < D / 32) sits at
-  // c * 32 + l, so that the 64-bit updates of a warp hit consecutive words
-  long long* acc = reinterpret_cast<long long*>(bmat + 2 * C::bmat_bytes(nbp));
-  float* cent_sm = reinterpret_cast<float*>(acc + 2 * cells);                     // [2][nb][D]
-  double* sums_sm = reinterpret_cast<double*>(cent_sm + 2 * cells);               // [nb][D]
+  unsigned char* stage_smem = base;                                               // [n_stages][kBoxes][128 x 128 B]
+  unsigned char* small_smem = base + static_cast<size_t>(n_stages) * C::kStageBytes;  // [kGroups][kBoxes][128 x 128 B]
+  unsigned char* hot_smem = small_smem + kGroups * C::kStageBytes;                // [kGroups][2][NBO x 128 B]
+  unsigned char* bmat = hot_smem + kGroups * C::kHotBytes;                        // [2][kBoxes][2 nbp x 128 B]
+  int* xchg = reinterpret_cast<int*>(bmat + 2 * C::bmat_bytes(nbp));  // d = 64: [NBO][64]
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < n_stages; ++i) {
       mbar_init(&full_bar[i], 1);
       mbar_init(&empty_bar[i], 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kDots; ++i) {
       mbar_init(&accfull[i], 1);
-      mbar_init(&accfree[i], 4);  // the four screening warps
+      mbar_init(&accfree[i], 4);  // the four warps of the tile's group
+    }
+    for (int i = 0; i < 2; ++i) {
       mbar_init(&bready[i], 1);
       mbar_init(&bfree[i], 1);
-      mbar_init(&accdone[i], 1);
-      mbar_init(&accclear[i], 1);
-      mbar_init(&cbar[i], 1);
-      mbar_init(&sfull[i], 1);
-      mbar_init(&sempty[i], 1);
     }
-    mbar_init(&sbar, 1);
-    mbar_init(&drain_bar, 1);
+    for (int i = 0; i < kGroups; ++i) {
+      mbar_init(&sumready[i], 4);
+      mbar_init(&smallfree[i], 1);
+    }
+    for (int i = 0; i < kSums; ++i) {
+      mbar_init(&sumfull[i], 1);
+      mbar_init(&cntready[i], 1);
+      mbar_init(&sumfree[i], 8);
+    }
+    mbar_init(&drain_bar[0], 1);
+    mbar_init(&drain_bar[1], 1);
     abort_sh = 0;
-    n_refine[0] = n_refine[1] = 0;
+    seen_sh = 0;
     fence_mbar_init();
   }
-  for (int c = threadIdx.x; c < 2 * cells; c += kUThreads) acc[c] = 0;
-  if (threadIdx.x < 2 * kMaxBeacons) add_cnt[threadIdx.x >> 5][threadIdx.x & 31] = 0;
+  for (uint32_t i = threadIdx.x; i < kGroups * C::kHotBytes / 16; i += kUThreads)
+    reinterpret_cast<uint4*>(hot_smem)[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = threadIdx.x; i < kSlots * kMaxBeacons; i += kUThreads) (&add_cnt[0][0])[i] = 0;
+  if (threadIdx.x < kSlots) spilled_sh[threadIdx.x] = 0;
+  if (threadIdx.x < kSpillSlots) list_sh[threadIdx.x].n = 0;
   if (warp == 1) {
     tmem_alloc(&tmem_base_sh, 512);
     tmem_relinquish();
   }
+  fence_proxy_async_smem();  // the one-hot operands' zeros are read by the tensor cores
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base_sh;
+  const uint32_t tmem_sums = tmem + kDots * ncols1;  // [kSums][kParts * NBO]
   volatile int* abort_flag = &abort_sh;
 
   if (warp == 0) {
     // ---------------------------------------------------------------- producer
-    if (lane == 0 && n_my > 0) {
+    if (elect_one()) {
       const uint64_t once = l2_policy_evict_first();
       prefetch_tmap(&qmap);
-      int g = 0;
+      int st = 0, round = 0;  // stage and how often the ring has gone round
       bool ok = true;
       for (int i = 0; ok && i < n_my; ++i) {
-        const int e = blockIdx.x + i * gridDim.x;
-        for (int t = 0; t < T; ++t, ++g) {
-          const int st = g % n_stages;
-          if (g >= n_stages &&
-              !mbar_wait(&empty_bar[st], ((g / n_stages) - 1) & 1, abort_flag, a.err, kDevTimeoutProducer)) {
+        const int row0 = (blockIdx.x + i * gridDim.x) * nq;
+        for (int t = 0; t < T; ++t) {
+          if (round > 0 && !mbar_wait(&empty_bar[st], (round - 1) & 1, abort_flag, a.err, kDevTimeoutProducer)) {
             ok = false;
             break;
           }
           mbar_arrive_expect_tx(&full_bar[st], static_cast<uint32_t>(C::kBoxes * a.box_rows * 128));
           for (int b = 0; b < C::kBoxes; ++b)
-            tma_load_2d(stage_smem + st * C::kStageBytes + b * kQBox, &qmap, &full_bar[st], b * 64,
-                        e * nq + t * kQTile, once);
+            tma_load_2d(stage_smem + st * C::kStageBytes + b * kQBox, &qmap, &full_bar[st], b * 64, row0 + t * kQTile,
+                        once);
+          if (++st == n_stages) {
+            st = 0;
+            ++round;
+          }
         }
       }
-      if (!ok || *abort_flag)
+      if (!ok || *abort_flag) {  // let every copy already issued land before the CTA exits
+        const int g = round * n_stages + st;
         for (int j = (g > n_stages ? g - n_stages : 0); j < g; ++j)
           drain_wait(&full_bar[j % n_stages], (j / n_stages) & 1, a.err);
+      }
     }
     __syncwarp();
   } else if (warp == 1) {
-    // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0 && n_my > 0) {
-      const uint32_t idesc1 = idesc_bf16_f32(128, ncols1), idesc2 = idesc_bf16_f32(128, kQTile);
-      int g = 0;
-      bool ok = true;
-      for (int i = 0; ok && i < n_my; ++i) {
-        const int pb = i & 1;
-        if (!mbar_wait(&bready[pb], (i >> 1) & 1, abort_flag, a.err, kDevTimeoutMma)) break;
-        for (int t = 0; t < T; ++t, ++g) {
-          const int st = g % n_stages, ab = g & 1;
-          if (!mbar_wait(&full_bar[st], (g / n_stages) & 1, abort_flag, a.err, kDevTimeoutMma) ||
-              (g >= 2 && !mbar_wait(&accfree[ab], ((g >> 1) - 1) & 1, abort_flag, a.err, kDevTimeoutMma))) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t d = tmem + ab * acc_cols;
-          const uint32_t q_addr = smem_u32(stage_smem + st * C::kStageBytes);
-          const uint32_t b_addr = smem_u32(bmat + pb * C::bmat_bytes(nbp));
+    // ---------------------------------------------------------------- screening MMAs
+    // Their own warp, so that a tile's dots never wait behind an earlier tile whose sums are not ready.
+    if (elect_one()) {
+      const uint32_t idesc1 = idesc_bf16_f32(128, ncols1);
+      const uint32_t stage0 = smem_u32(stage_smem);
+      int si = 0, s_t = 0, s_st = 0, s_round = 0, s_ab = 0, s_use = 0;  // screening: instance, tile, stage, accumulator
+      auto screen = [&]() -> bool {
+        const int pb = si & 1;
+        if (s_t == 0 && !mbar_wait(&bready[pb], (si >> 1) & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
+        if (!mbar_wait(&full_bar[s_st], s_round & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
+        if (s_use > 0 && !mbar_wait(&accfree[s_ab], (s_use - 1) & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
+        tc_fence_after();
+        const uint32_t d = tmem + s_ab * ncols1;
+        const uint32_t q_addr = stage0 + s_st * C::kStageBytes;
+        const uint32_t b_addr = smem_u32(bmat) + pb * C::bmat_bytes(nbp);
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint32_t qoff = (kk >> 2) * kQBox + (kk & 3) * 32;
-            const uint32_t boff = (kk >> 2) * bbox + (kk & 3) * 32;
-            mma_bf16_ss(d, sdesc_kmajor_sw128(q_addr + qoff), sdesc_kmajor_sw128(b_addr + boff), idesc1, kk > 0);
-          }
-#pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint32_t qoff = (kk >> 2) * kQBox + (kk & 3) * 32;
-            mma_bf16_ss(d + ncols1, sdesc_kmajor_sw128(q_addr + qoff), sdesc_kmajor_sw128(q_addr + qoff), idesc2,
-                        kk > 0);
-          }
-          mma_commit(&accfull[ab]);
+        for (int kk = 0; kk < D / 16; ++kk)
+          mma_bf16_ss(d, sdesc_kmajor_sw128(q_addr + (kk >> 2) * kQBox + (kk & 3) * 32),
+                      sdesc_kmajor_sw128(b_addr + (kk >> 2) * bbox + (kk & 3) * 32), idesc1, kk > 0);
+        mma_commit(&accfull[s_ab]);
+        if (++s_t == T) {
+          mma_commit(&bfree[pb]);  // this instance's centroid operand is no longer read
+          s_t = 0;
+          ++si;
         }
-        if (ok) mma_commit(&bfree[pb]);  // this instance's centroid operand is no longer read
-      }
-      mma_commit(&drain_bar);
-      drain_wait(&drain_bar, 0, a.err);
+        if (++s_st == n_stages) {
+          s_st = 0;
+          ++s_round;
+        }
+        if (++s_ab == kDots) {
+          s_ab = 0;
+          ++s_use;
+        }
+        return true;
+      };
+      for (int g = 0; g < n_tiles; ++g)
+        if (!screen()) break;
+      mma_commit(&drain_bar[0]);
+      drain_wait(&drain_bar[0], 0, a.err);
     }
     __syncwarp();
-  } else if (warp < 2 + kScreeners) {
-    // ---------------------------------------------------------------- screeners
-    const int ws = warp - 2;          // 0 .. 3
-    const int quarter = warp & 3;     // TMEM lane quarter (warps 2..5 cover all four)
-    const int ts = threadIdx.x - 64;  // 0 .. 127
-    const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
-    const int n = quarter * 32 + lane;  // this thread's query row in the tile
-    const int col0 = lane * kCols;
-    const unsigned lt = (1u << lane) - 1u;
-    int g = 0;
-    for (int i = 0; i < n_my; ++i) {
-      const int e = blockIdx.x + i * gridDim.x;
-      const int pb = i & 1;
-      long long* acc_i = acc + pb * cells;
-      const float* cent_i = cent_sm + pb * cells;
-      // re-decided rows go straight into acc_i: wait until the fold two instances back cleared it
-      if (i >= 2) mbar_wait(&accclear[pb], ((i >> 1) - 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
-      for (int t = 0; t < T; ++t, ++g) {
-        const int st = g % n_stages, ab = g & 1, ob = g & 1;
-        const int rows = min(kQTile, nq - t * kQTile);
-        const unsigned char* qs = stage_smem + st * C::kStageBytes;
-        int* assign_t = a.assign_out ? a.assign_out + static_cast<size_t>(e) * nq + t * kQTile : nullptr;
-
-        // ---- dots and norm of this thread's query from tensor memory
-        bool have = !*abort_flag && mbar_wait(&accfull[ab], (g >> 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
-        have = __all_sync(0xffffffffu, have);
-        float best = -INFINITY, second = -INFINITY, qn2 = 0.f;
-        int bi = -1;
-        bool any_valid = false;  // a valid beacon (screened values that are all NaN leave bi at -1)
-        if (have) {
-          tc_fence_after();
-          const uint32_t d = tmem + ab * acc_cols + lane_addr;
-          float v[32];
-          tmem_ld32(d + ncols1 + quarter * 32, v);  // Q Q^T columns of this quarter: the diagonal is v[lane]
-          tmem_wait_ld();
+  } else if (warp == 2) {
+    // ---------------------------------------------------------------- sum MMAs
+    if (elect_one()) {
+      const uint32_t idesc2 = idesc_bf16_f32(128, NBO) | (1u << 15);  // A is read across its rows
+      const uint32_t stage0 = smem_u32(stage_smem);
+      int m_st = 0;  // stage
+      auto sum = [&](int g) -> bool {
+        const int sb = g % kGroups, ub = g % kSums;
+        if (!mbar_wait(&sumready[sb], (g / kGroups) & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
+        if (g >= kSums && !mbar_wait(&sumfree[ub], ((g / kSums) - 1) & 1, abort_flag, a.err, kDevTimeoutMma))
+          return false;
+        // passes on what the group wrote besides the operands; after the wait above, so that the barrier is
+        // never two phases ahead of the warps that wait for it
+        mbar_arrive(&cntready[ub]);
+        tc_fence_after();
+        const uint32_t d = tmem_sums + ub * (C::kParts * NBO);
+        const uint32_t q_addr = stage0 + m_st * C::kStageBytes;
+        const uint32_t s_addr = smem_u32(small_smem) + sb * C::kStageBytes;
+        const uint32_t h_addr = smem_u32(hot_smem) + sb * C::kHotBytes;
+        // A: 128 "rows" are the columns of d (d = 64: the tile's 64, then the second tile's 64)
+        const uint32_t lbo = D == 128 ? kQBox : s_addr - q_addr;
+        // the second tile's product first: its group waits for that buffer longest
 #pragma unroll
-          for (int k = 0; k < 32; ++k) qn2 = (k == lane) ? v[k] : qn2;
+        for (int p = C::kParts - 1; p >= 0; --p) {
+#pragma unroll
+          for (int kk = 0; kk < kQTile / 16; ++kk)
+            mma_bf16_ss(d + p * NBO, sdesc_mnmajor_sw128((p ? s_addr : q_addr) + kk * 2048, lbo),
+                        sdesc_kmajor_sw128(h_addr + (kk >> 2) * (NBO * 128) + (kk & 3) * 32), idesc2, kk > 0);
+          if (p == C::kParts - 1) mma_commit(&smallfree[sb]);
+        }
+        mma_commit(&sumfull[ub]);
+        mma_commit(&empty_bar[m_st]);  // the stage's queries are no longer read
+        if (++m_st == n_stages) m_st = 0;
+        return true;
+      };
+      for (int g = 0; g < n_tiles; ++g)
+        if (!sum(g)) break;
+      mma_commit(&drain_bar[1]);
+      drain_wait(&drain_bar[1], 0, a.err);
+    }
+    __syncwarp();
+  } else if (warp < kSumWarp0) {
+    // ---------------------------------------------------------------- row groups: one query per thread
+    const int sb = (warp - kGroupWarp0) >> 2;  // this group: tiles sb, sb + kGroups, ...
+    const int quarter = warp & 3;        // TMEM lane quarter
+    const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
+    const int n = quarter * 32 + lane;   // this thread's query in the tile
+    const uint32_t swz = static_cast<uint32_t>(n & 7) << 4;
+    unsigned char* small_row = small_smem + sb * C::kStageBytes + n * 128;
+    unsigned char* hot = hot_smem + sb * C::kHotBytes + (n >> 6) * (NBO * 128) + ((n & 7) << 1);
+    const uint32_t hot_chunk = static_cast<uint32_t>((n & 63) >> 3);
+    int prev_b = -1;                     // beacon whose cell of the one-hot column is set
+    int i = 0, t = sb;
+    while (t >= T) {
+      t -= T;
+      ++i;
+    }
+    for (int g = sb; g < n_tiles; g += kGroups) {
+      const int e = blockIdx.x + i * gridDim.x;
+      const int st = g % n_stages, ab = g % kDots, slot = i & (kSlots - 1);
+      const int rows = min(kQTile, nq - t * kQTile);
+      // the tile's data and its dots (which also says that the screening has read the tile)
+      bool ok = mbar_wait(&full_bar[st], (g / n_stages) & 1, abort_flag, a.err, kDevTimeoutEpilogue) &&
+                mbar_wait(&accfull[ab], (g / kDots) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      tc_fence_after();
+      const int E = static_cast<signed char>(exp_sh[slot] & 0xff);
+      const bool degenerate = (exp_sh[slot] & 0x100) != 0;
+      const uint32_t vm = vmask_sh[slot];
+
+      // ---- best and second best dot
+      const uint32_t d = tmem + ab * ncols1 + lane_addr;
+      float best = -INFINITY, second = -INFINITY;
+      int bi = -1;
+      for (int c0 = 0; c0 < nbp; c0 += 8) {
+        float h[8], l[8];
+        tmem_ld8(d + c0, h);
+        tmem_ld8(d + nbp + c0, l);
+        tmem_wait_ld();
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const float dot = ((vm >> (c0 + u)) & 1u) ? h[u] + l[u] : -INFINITY;
+          second = fmaxf(second, fminf(best, dot));
+          if (dot > best) {
+            best = dot;
+            bi = c0 + u;
+          }
+        }
+      }
+
+      // this group's second tile is free once its previous tile's product is formed (the one-hot operand: below)
+      ok = g < kGroups || mbar_wait(&smallfree[sb], ((g / kGroups) - 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
+      if (!__all_sync(0xffffffffu, ok)) break;
+
+      // ---- the split of this query's elements, its squared norm and its extremes
+      unsigned char* raw_row = stage_smem + st * C::kStageBytes + n * 128;
+      uint32_t below = 0u;                 // bits of the elements below the operands' range
+      float qn2 = 0.f;
+      if (n < rows) {
+        const __nv_bfloat162 lim = as_bf162(pow2_bf16x2(E - kLargeBits));
+        const __nv_bfloat162 lim_lo = as_bf162(pow2_bf16x2(E - kSmallBits));
+        __nv_bfloat162 n2[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) n2[k] = as_bf162(0u);
+        // four chunks are loaded before the first store: a chunk at a time would wait out its latencies
+        // (rolled in between: the roles of this kernel compete for the instruction caches)
+#pragma unroll 1
+        for (int c0 = 0; c0 < D / 8; c0 += 4) {
+          unsigned char* box_raw = raw_row + (c0 >> 3) * kQBox;
+          unsigned char* box_small = small_row + (c0 >> 3) * kQBox;
+          uint4 v[4];
+          uint32_t off[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            off[c] = static_cast<uint32_t>(((c0 & 4) + c) << 4) ^ swz;
+            v[c] = *reinterpret_cast<const uint4*>(box_raw + off[c]);
+          }
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const uint32_t w[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
+            uint32_t s[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const __nv_bfloat162 x2 = as_bf162(w[k]), a2 = __habs2(x2);
+              s[k] = w[k] & __hlt2_mask(a2, lim);
+              below |= w[k] & __hlt2_mask(a2, lim_lo);
+              n2[k] = __hfma2(x2, x2, n2[k]);
+            }
+            *reinterpret_cast<uint4*>(box_small + off[c]) = make_uint4(s[0], s[1], s[2], s[3]);
+            st_shared_v4_if((s[0] | s[1]) | (s[2] | s[3]), box_raw + off[c], w[0] ^ s[0], w[1] ^ s[1], w[2] ^ s[2],
+                            w[3] ^ s[3]);
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float2 f = __bfloat1622float2(n2[k]);
+          qn2 += f.x + f.y;
+        }
+      } else {  // no query: nothing of a neighbour or of an earlier tile may enter the sums
+        const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+        for (int c = 0; c < D / 8; ++c) {
+          const uint32_t off = (c >> 3) * kQBox + (static_cast<uint32_t>((c & 7) << 4) ^ swz);
+          *reinterpret_cast<uint4*>(raw_row + off) = z;
+          *reinterpret_cast<uint4*>(small_row + off) = z;
+        }
+      }
+      qn2 *= 1.1f;  // within a few percent (16 bf16 roundings per sum): taken too large
+      // |q| < 2^E bounds every element
+      const bool special = !(qn2 < __uint_as_float(static_cast<uint32_t>(2 * E + 127) << 23)) || (below & 0x7fff7fffu) != 0u;
+      {
+        const uint32_t wmx =
+            __reduce_max_sync(0xffffffffu, qn2 < static_cast<float>(1 << (2 * kMaxE)) ? __float_as_uint(qn2) : 0u);
+        if (lane == 0 && wmx > *reinterpret_cast<volatile uint32_t*>(&seen_sh)) atomicMax(&seen_sh, wmx);
+      }
+
+      // ---- decision
+      const bool wild = degenerate || !(qn2 > 1e-30f && qn2 < 1e30f);
+      const float margin = kMarginRel * sqrt_approx(qn2);
+      const bool close = n < rows && vm != 0u && (wild || !(best - second > margin));
+      int my_b = n < rows ? bi : -1;
+      uint32_t need = __ballot_sync(0xffffffffu, close);
+      if (need) {  // rare: which beacons may be the exact best, while the dots are still there
+        uint32_t cand = vm;
+        if (!__all_sync(0xffffffffu, !close || wild)) {
+          const float floor_v = best - 2.f * margin;
+          uint32_t m = 0u;
           for (int c0 = 0; c0 < nbp; c0 += 8) {
-            uint32_t h[8], l[8];
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                : "=r"(h[0]), "=r"(h[1]), "=r"(h[2]), "=r"(h[3]), "=r"(h[4]), "=r"(h[5]), "=r"(h[6]), "=r"(h[7])
-                : "r"(d + c0));
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                : "=r"(l[0]), "=r"(l[1]), "=r"(l[2]), "=r"(l[3]), "=r"(l[4]), "=r"(l[5]), "=r"(l[6]), "=r"(l[7])
-                : "r"(d + nbp + c0));
+            float h[8], l[8];
+            tmem_ld8(d + c0, h);
+            tmem_ld8(d + nbp + c0, l);
             tmem_wait_ld();
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              const int b = c0 + u;
-              if (b < nb && bvalid[pb][b]) {
-                any_valid = true;
-                const float dot = __uint_as_float(h[u]) + __uint_as_float(l[u]);
-                if (dot > best) {
-                  second = best;
-                  best = dot;
-                  bi = b;
-                } else if (dot > second) {
-                  second = dot;
-                }
-              }
-            }
+            for (int u = 0; u < 8; ++u) m |= (h[u] + l[u] >= floor_v ? 1u : 0u) << (c0 + u);
           }
+          if (!wild) cand = m & vm;
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&accfree[ab]);
+        for (uint32_t m = need; m; m &= m - 1) {
+          const int r = __ffs(m) - 1;
+          __syncwarp();  // the rows' splits are written
+          const int b = refine_row<D>(stage_smem + st * C::kStageBytes, small_smem + sb * C::kStageBytes, quarter * 32 + r,
+                                      a.cent + static_cast<size_t>(e) * nb * D, __shfl_sync(0xffffffffu, cand, r));
+          if (lane == r) my_b = b;
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&accfree[ab]);
 
-        // ---- decision; close calls go to the exact list; counts per beacon by ballot
-        int my_b = -1, my_pos = 0;
-        if (have && n < rows) {
-          if (any_valid && (degenerate[pb] || !(qn2 > 1e-30f && qn2 < 1e30f) ||
-                          !(best - second > kMarginRel * sqrtf(qn2)))) {
-            refine_t[ob][atomicAdd(&n_refine[ob], 1)] = n;
-          } else {
-            my_b = bi;
-            if (assign_t) assign_t[n] = bi;
-          }
-        }
-        for (int b = 0; b < nb; ++b) {
-          const unsigned m = __ballot_sync(0xffffffffu, my_b == b);
-          if (lane == b) cnt_w[ob][quarter][b] = __popc(m);
-          if (my_b == b) my_pos = __popc(m & lt);
-        }
-        named_barrier(1, 32 * kScreeners);
-
-        // ---- sorted row list for the accumulators (its buffer is free once they are done with tile g - 2)
-        if (g >= 2) mbar_wait(&sempty[ob], ((g >> 1) - 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
-        if (ts == 0) n_refine[ob ^ 1] = 0;  // the next tile's list; its previous readers finished a tile ago
-        {
-          int tot = 0, mine = 0;
-          if (lane < nb)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int c = cnt_w[ob][q][lane];
-              tot += c;
-              mine += (q < quarter) ? c : 0;
-            }
-          int incl = tot;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-          }
-          const int off = incl - tot + mine;  // where this warp's rows of beacon `lane` start
-          const int my_off = __shfl_sync(0xffffffffu, off, my_b < 0 ? 0 : my_b);
-          if (my_b >= 0) order_t[ob][my_off + my_pos] = n | (my_b << 8);
-          if (quarter == 0) {
-            if (lane == 31) n_asg_sh[ob] = incl;
-            if (lane < nb && tot > 0) atomicAdd(&add_cnt[pb][lane], tot);  // refinements add concurrently
-          }
-        }
-
-        // ---- exact decisions for close calls, one warp per query; the row is added here
-        const int nr = n_refine[ob];
-        for (int k = ws; k < nr; k += kScreeners) {
-          const int r = refine_t[ob][k];
-          float x[D / 32];
-#pragma unroll
-          for (int j = 0; j < D / 32; ++j)
-            x[j] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(qs + sw128_offset(r, lane + 32 * j, kQBox)));
-          const int best_b = exact_decision<D>(
-              x, nb, [&](int b, int col) { return cent_i[b * D + col]; }, [&](int b) { return bvalid[pb][b] != 0; },
-              cninv[pb]);
-          if (lane == 0) {
-            if (assign_t) assign_t[r] = best_b;
-            if (best_b >= 0) atomicAdd(&add_cnt[pb][best_b], 1);
-          }
-          if (best_b >= 0) {
-            long long sr[kCols];
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) sr[c] = 0;
-            add_fixed<kCols>(sr, qs + sw128_offset(r, col0, kQBox));
-#pragma unroll
-            for (int c = 0; c < kCols; ++c)
-              shared_add_i64(&acc_i[best_b * D + c * 32 + lane], sr[c]);
-          }
-        }
-        named_barrier(1, 32 * kScreeners);
-        if (ts == 0) mbar_arrive(&sfull[ob]);
+      if (n < rows && a.assign_out) a.assign_out[static_cast<size_t>(e) * nq + t * kQTile + n] = my_b;
+      add_counts<NBO>(add_cnt[slot], my_b);
+      ok = g < kGroups || mbar_wait(&sumfull[(g - kGroups) % kSums], ((g - kGroups) / kSums) & 1, abort_flag, a.err,
+                                    kDevTimeoutEpilogue);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      // ---- this query's column of the one-hot operand: 2^(17 - E), which makes the large part's sums integers
+      if (prev_b >= 0) *reinterpret_cast<uint16_t*>(hot + prev_b * 128 + ((hot_chunk ^ (prev_b & 7)) << 4)) = 0;
+      if (my_b >= 0)
+        *reinterpret_cast<uint16_t*>(hot + my_b * 128 + ((hot_chunk ^ (my_b & 7)) << 4)) =
+            static_cast<uint16_t>(pow2_bf16x2(kLargeBits + 7 - E));
+      prev_b = my_b;
+      for (uint32_t m = __ballot_sync(0xffffffffu, special); m; m &= m - 1) {  // rare
+        const int r = __ffs(m) - 1, b = __shfl_sync(0xffffffffu, my_b, r);
+        const int si = i & (kSpillSlots - 1);
+        __syncwarp();  // the rows' splits are written
+        if (spill_row<D>(stage_smem + st * C::kStageBytes, small_smem + sb * C::kStageBytes, quarter * 32 + r, E, b,
+                         &list_sh[si], a.spill + (static_cast<size_t>(blockIdx.x) * kSpillSlots + si) * nb * D))
+          spilled_sh[slot] = 1;
+      }
+      fence_proxy_async_smem();  // this thread's operand writes, read next by the tensor cores
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sumready[sb]);
+      t += kGroups;
+      while (t >= T) {
+        t -= T;
+        ++i;
       }
     }
-  } else if (warp < 2 + kScreeners + kAccum) {
-    // ---------------------------------------------------------------- accumulators
-    const int wa = warp - 2 - kScreeners;               // 0 .. kAccum - 1
-    const int ta = threadIdx.x - 32 * (2 + kScreeners);  // 0 .. 32 * kAccum - 1
-    const int col0 = lane * kCols;
-    const int chunk = (col0 & 63) >> 3;
-    const uint32_t lane_off = (col0 >> 6) * kQBox + ((col0 & 7) << 1);
-    int g = 0;
-    for (int i = 0; i < n_my; ++i) {
-      const int pb = i & 1;
-      long long* acc_i = acc + pb * cells;
-      if (i >= 2) mbar_wait(&accclear[pb], ((i >> 1) - 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
-      for (int t = 0; t < T; ++t, ++g) {
-        const int st = g % n_stages, ob = g & 1;
-        const unsigned char* qs = stage_smem + st * C::kStageBytes + lane_off;
-        const bool ready = mbar_wait(&sfull[ob], (g >> 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
-        const int n_asg = ready ? n_asg_sh[ob] : 0;
-        const int* ord = order_t[ob];
-        const int p1 = (wa + 1) * n_asg / kAccum;
-        int p = wa * n_asg / kAccum;
-        auto row_ptr = [&](int en) {
-          const int r = en & 0xff;
-          return qs + r * 128 + ((chunk ^ (r & 7)) << 4);
-        };
-        constexpr int kPairs = kCols / 2;
-        Parts2 s[kPairs];
+  } else if (warp < kBuildWarp0) {
+    // ---------------------------------------------------------------- sums: a column of d and half of the beacons
+    // per thread (two warps per TMEM lane quarter)
+    constexpr int HB = NBO / 2;
+    const int quarter = warp & 3;
+    const int h0 = ((warp - kSumWarp0) >> 2) * HB;  // first beacon
+    const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
+    const int col = quarter * 32 + lane;        // d = 64: 64 and more are the small parts of column col - 64
+    const bool small_half = D == 64 && col >= 64;
+    const bool first_warp = warp == kSumWarp0;
+    for (int i = 0, g = 0; i < n_my; ++i) {
+      const int e = blockIdx.x + i * gridDim.x, slot = i & (kSlots - 1);
+      const size_t cells = static_cast<size_t>(nb) * D, cbase = static_cast<size_t>(e) * cells;
+      if (first_warp && lane == 0) bulk_prefetch_l2(a.sums + cbase, static_cast<uint32_t>(cells) * 8);
+      // sums of the two operands, each below 2^24 per tile (d = 64: of one, by this thread's half); more than
+      // kFlush tiles are passed on through the spill array
+      constexpr int kFlush = 64;
+      int acc_l[HB], acc_s[HB];
 #pragma unroll
-        for (int h = 0; h < kPairs; ++h) s[h] = Parts2{0ull, 0ull, 0ull};
-        int cur = -1;
-        auto flush = [&]() {
+      for (int b = 0; b < HB; ++b) acc_l[b] = acc_s[b] = 0;
+      const long long cnt_old = lane < nb ? a.counts[static_cast<size_t>(e) * nb + lane] : 0;
+      bool ok = true;  // false after a wait gave up: the barriers below are still taken
+      constexpr int kChunk = 2;  // beacons folded at once (more would overlap more latency, but cost instruction cache)
+      double s_old[kChunk];      // running sums of the next chunk to fold
+      auto load_old = [&](int b0) {
 #pragma unroll
-          for (int c = 0; c < kCols; ++c)
-            shared_add_i64(&acc_i[cur * D + c * 32 + lane], fixed40(parts2_get(s[c >> 1], c & 1)));
+        for (int u = 0; u < kChunk; ++u)
+          s_old[u] = b0 + u < nb && !small_half ? a.sums[cbase + static_cast<size_t>(b0 + u) * D + col] : 1.0;
+      };
+      for (int t = 0; ok && t < T; ++t, ++g) {
+        const int ub = g % kSums;
+        if (t == T - 1) load_old(h0);  // ahead of the last tile's sums
+        ok = mbar_wait(&cntready[ub], (g / kSums) & 1, abort_flag, a.err, kDevTimeoutEpilogue) &&
+             mbar_wait(&sumfull[ub], (g / kSums) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d = tmem_sums + ub * (C::kParts * NBO) + lane_addr + h0;
+        // large sums are integers (the one-hot operand's scale), small ones multiples of 2^-10
 #pragma unroll
-          for (int h = 0; h < kPairs; ++h) s[h] = Parts2{0ull, 0ull, 0ull};
-        };
-        auto add_row = [&](const unsigned char* rp) {
-          if constexpr (kCols == 4) {
-            const uint2 v = *reinterpret_cast<const uint2*>(rp);
-            parts2_add(s[0], v.x);
-            parts2_add(s[1 % kPairs], v.y);
-          } else {
-            parts2_add(s[0], *reinterpret_cast<const uint32_t*>(rp));
+        for (int b0 = 0; b0 < HB; b0 += 8) {
+          float v[C::kParts][8];
+#pragma unroll
+          for (int p = 0; p < C::kParts; ++p) tmem_ld8(d + p * NBO + b0, v[p]);
+          tmem_wait_ld();
+          if (b0 + 8 == HB) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sumfree[ub]);
           }
-        };
-        while (p < p1) {
-          if (p + kGroup <= p1 && (ord[p] >> 8) == cur && (ord[p + kGroup - 1] >> 8) == cur) {
-            // sorted: the group's rows share the beacon
 #pragma unroll
-            for (int r = 0; r < kGroup; ++r) add_row(row_ptr(ord[p + r]));
-            p += kGroup;
-            continue;
+          for (int b = 0; b < 8; ++b) {
+            if constexpr (D == 128) {
+              acc_l[b0 + b] += __float2int_rn(v[0][b]);
+              acc_s[b0 + b] += __float2int_rn(v[C::kParts - 1][b] * 1024.f);
+            } else {
+              acc_l[b0 + b] += __float2int_rn(small_half ? v[0][b] * 1024.f : v[0][b]);
+            }
           }
-          const int en = ord[p];
-          const int b = en >> 8;
-          if (b != cur) {
-            if (cur >= 0) flush();
-            cur = b;
-          }
-          add_row(row_ptr(en));
-          ++p;
         }
-        if (cur >= 0) flush();
-        named_barrier(2, 32 * kAccum);
-        if (ta == 0) {
-          mbar_arrive(&empty_bar[st]);  // the stage's queries are no longer read
-          mbar_arrive(&sempty[ob]);
-          if (t == T - 1) mbar_arrive(&accdone[pb]);  // this instance's sums are complete
+        if (t + 1 < T && (t + 1) % kFlush == 0) {  // rare: more than 8192 queries per instance
+          const int shift = static_cast<signed char>(exp_sh[slot] & 0xff) + 40 - (kSmallBits + 7);
+          unsigned long long* sp =
+              a.spill + (static_cast<size_t>(blockIdx.x) * kSpillSlots + (i & (kSpillSlots - 1))) * cells;
+#pragma unroll
+          for (int b = 0; b < HB; ++b) {
+            const long long f = (D == 128 ? acc_l[b] * 1024ll + acc_s[b] : small_half ? acc_l[b] : acc_l[b] * 1024ll)
+                                << shift;
+            if (h0 + b < nb && f != 0)
+              atomicAdd(sp + (h0 + b) * D + (small_half ? col - 64 : col), static_cast<unsigned long long>(f));
+            acc_l[b] = acc_s[b] = 0;
+          }
+          spilled_sh[slot] = 1;
+          __threadfence();
         }
+      }
+      if (T > kFlush) named_barrier(1, 256);  // what another warp passed on (d = 64) is there
+
+      // ---- fold this instance's sums into the running state
+      const int add = lane < nb ? add_cnt[slot][lane] : 0;
+      const uint32_t touched = ok ? __ballot_sync(0xffffffffu, add > 0) : 0u;
+      const DF rcp = count_reciprocal(add > 0 ? cnt_old + add : 1);  // lane b: beacon b
+      const int shift = static_cast<signed char>(exp_sh[slot] & 0xff) + 40 - (kSmallBits + 7);  // to units of 2^-40
+      const bool spilled = spilled_sh[slot] != 0;
+      const SpillList& list = list_sh[i & (kSpillSlots - 1)];
+      const int n_list = min(list.n, kSpillList);
+      unsigned long long* spill =
+          a.spill + (static_cast<size_t>(blockIdx.x) * kSpillSlots + (i & (kSpillSlots - 1))) * cells;
+      if constexpr (D == 64) {
+        if (small_half)
+#pragma unroll
+          for (int b = 0; b < HB; ++b) xchg[(h0 + b) * 64 + col - 64] = acc_l[b];
+        named_barrier(1, 256);
+        if (!small_half)
+#pragma unroll
+          for (int b = 0; b < HB; ++b) acc_s[b] = xchg[(h0 + b) * 64 + col];
+      }
+#pragma unroll 1
+      for (int b0 = h0; b0 < nb && b0 < h0 + HB; b0 += kChunk) {  // chunk b0 sits in acc_*[0 .. kChunk)
+        double s_in[kChunk];
+        long long f[kChunk];
+        bool mine[kChunk];
+#pragma unroll
+        for (int u = 0; u < kChunk; ++u) {
+          const int b = b0 + u;
+          mine[u] = b < nb && ((touched >> (b & 31)) & 1u) && !small_half;
+          s_in[u] = mine[u] ? s_old[u] : 1.0;
+          f[u] = mine[u] ? (acc_l[u] * 1024ll + acc_s[u]) << shift : 0;
+          if (mine[u] && spilled) {
+            f[u] += static_cast<long long>(__ldcg(spill + b * D + col));
+            spill[b * D + col] = 0ull;
+          }
+        }
+        if (b0 + kChunk < h0 + HB) load_old(b0 + kChunk);
+        for (int k = 0; k < n_list; ++k) {
+          const int rel = list.key[k] - ((b0 << 8) | col);  // (beacon - b0) << 8 where the column is this thread's
+#pragma unroll
+          for (int u = 0; u < kChunk; ++u)
+            if (rel == u << 8 && mine[u]) f[u] += list.val[k];
+        }
+        // the common case for the chunk at once (the cells' latencies overlap), the rest one by one
+        double s_new[kChunk];
+        float c_new[kChunk];
+        bool plain = true;
+#pragma unroll
+        for (int u = 0; u < kChunk; ++u) {
+          const int b = (b0 + u) & 31;
+          const DF rb{__shfl_sync(0xffffffffu, rcp.hi, b), __shfl_sync(0xffffffffu, rcp.lo, b)};
+          plain &= fold_and_centroid(s_in[u], f[u], rb, s_new[u], c_new[u]);
+        }
+        if (!plain) {
+#pragma unroll 1
+          for (int u = 0; u < kChunk; ++u) {
+            const int b = (b0 + u) & 31;
+            DF rb = count_reciprocal(1);
+            if (b < nb && add_cnt[slot][b] > 0) rb = count_reciprocal(a.counts[static_cast<size_t>(e) * nb + b] + add_cnt[slot][b]);
+            double so = s_in[0];
+            long long fu = f[0];
+#pragma unroll
+            for (int k = 1; k < kChunk; ++k) {
+              so = k == u ? s_in[k] : so;
+              fu = k == u ? f[k] : fu;
+            }
+            const double sn = fold_sum(so, fu);
+            const float cn = centroid_value(sn, rb);
+#pragma unroll
+            for (int k = 0; k < kChunk; ++k) {
+              s_new[k] = k == u ? sn : s_new[k];
+              c_new[k] = k == u ? cn : c_new[k];
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kChunk; ++u)
+          if (mine[u]) {
+            const size_t gi = cbase + static_cast<size_t>(b0 + u) * D + col;
+            a.sums[gi] = s_new[u];
+            a.cent[gi] = c_new[u];
+          }
+#pragma unroll
+        for (int b = 0; b + kChunk < HB; ++b) {
+          acc_l[b] = acc_l[b + kChunk];
+          acc_s[b] = acc_s[b + kChunk];
+        }
+      }
+      if (spilled) __threadfence();
+      named_barrier(1, 256);  // every warp has read this slot's words, the counts (and, d = 64, the exchanged sums)
+      if (ok && first_warp && add > 0) a.counts[static_cast<size_t>(e) * nb + lane] = cnt_old + add;
+      if (first_warp) add_cnt[slot][lane] = 0;
+      if (first_warp && lane == 0) {
+        spilled_sh[slot] = 0;
+        list_sh[i & (kSpillSlots - 1)].n = 0;
       }
     }
   } else {
-    // ---------------------------------------------------------------- bookkeeping
-    const int wk = warp - 2 - kScreeners - kAccum;  // 0 .. 3
-    const int tk = threadIdx.x - 32 * (2 + kScreeners + kAccum);
-    const uint32_t cbytes = static_cast<uint32_t>(cells) * 4, sbytes = static_cast<uint32_t>(cells) * 8;
-    auto inst = [&](int idx) { return blockIdx.x + idx * gridDim.x; };
-    auto issue_cent = [&](int idx) {  // centroids of instance idx into cent_sm[idx & 1]
-      fence_proxy_async_smem();
-      mbar_arrive_expect_tx(&cbar[idx & 1], cbytes);
-      bulk_copy_g2s(cent_sm + (idx & 1) * cells, a.cent + static_cast<size_t>(inst(idx)) * cells, cbytes,
-                    &cbar[idx & 1]);
-    };
-    auto issue_sums = [&](int idx) {
-      fence_proxy_async_smem();
-      mbar_arrive_expect_tx(&sbar, sbytes);
-      bulk_copy_g2s(sums_sm, a.sums + static_cast<size_t>(inst(idx)) * cells, sbytes, &sbar);
-    };
-    auto build = [&](int idx) {
-      const int pb = idx & 1;
-      const int e = inst(idx);
-      if (tk < nb) cnt_old[pb][tk] = a.counts[static_cast<size_t>(e) * nb + tk];
-      if (tk == 0) degenerate[pb] = 0;
-      mbar_wait(&cbar[pb], (idx >> 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
-      if (idx >= 2) mbar_wait(&bfree[pb], ((idx >> 1) - 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
-      named_barrier(3, 32 * kKeepers);
-      const float* cs = cent_sm + pb * cells;
+    // ---------------------------------------------------------------- builders: the unit-centroid operand
+    const int wk = warp - kBuildWarp0;  // 0 .. 3
+    constexpr int kBatch = 1;
+    for (int i = 0; i < n_my; ++i) {
+      const int e = blockIdx.x + i * gridDim.x, pb = i & 1, slot = i & (kSlots - 1);
+      if (wk == 0 && lane == 0 && i + 1 < n_my)
+        bulk_prefetch_l2(a.cent + (static_cast<size_t>(e) + gridDim.x) * nb * D, static_cast<uint32_t>(nb * D) * 4);
+      const long long cnt = lane < nb ? a.counts[static_cast<size_t>(e) * nb + lane] : 0;
+      const uint32_t counted = __ballot_sync(0xffffffffu, cnt > 0);
+      if (i >= 2) mbar_wait(&bfree[pb], ((i >> 1) - 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
       unsigned char* bm = bmat + pb * C::bmat_bytes(nbp);
-      for (int b = wk; b < nbp; b += kKeepers) {
-        float c[D / 32];
-        float n2 = 0.f;
-        DF n2d{0.f, 0.f};  // the exact products c^2 summed in double-float arithmetic
-        int nz = 0;
+      uint32_t valid = 0u;
+      float cmax = 0.f;
+      bool extreme = false;
+#pragma unroll 1
+      for (int b0 = wk; b0 < nbp; b0 += 4 * kBatch) {
+        float c[kBatch][D / 32];
 #pragma unroll
-        for (int k = 0; k < D / 32; ++k) {
-          c[k] = b < nb ? cs[b * D + lane + 32 * k] : 0.f;
-          n2 = fmaf(c[k], c[k], n2);
-          n2d = df_add(n2d, df_two_prod(c[k], c[k]));
-          nz |= (c[k] != 0.f);
-        }
+        for (int u = 0; u < kBatch; ++u)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          n2 += __shfl_xor_sync(0xffffffffu, n2, o);
-          nz |= __shfl_xor_sync(0xffffffffu, nz, o);
-        }
+          for (int k = 0; k < D / 32; ++k)
+            c[u][k] = b0 + 4 * u < nb ? a.cent[(static_cast<size_t>(e) * nb + b0 + 4 * u) * D + lane + 32 * k] : 0.f;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-          n2d = df_add(n2d, DF{__shfl_xor_sync(0xffffffffu, n2d.hi, o), __shfl_xor_sync(0xffffffffu, n2d.lo, o)});
-        const bool ok = b < nb && cnt_old[pb][b] > 0 && nz;
-        const float inv = ok ? rsqrtf(n2) : 0.f;
+        for (int u = 0; u < kBatch; ++u) {
+          const int b = b0 + 4 * u;
+          if (b >= nbp) break;
+          float n2 = 0.f;
 #pragma unroll
-        for (int k = 0; k < D / 32; ++k) {
-          const int col = lane + 32 * k;
-          const float u = c[k] * inv;
-          const __nv_bfloat16 hi = __float2bfloat16_rn(u);
-          const __nv_bfloat16 lo = __float2bfloat16_rn(u - __bfloat162float(hi));
-          *reinterpret_cast<__nv_bfloat16*>(bm + sw128_offset(b, col, bbox)) = hi;
-          *reinterpret_cast<__nv_bfloat16*>(bm + sw128_offset(nbp + b, col, bbox)) = lo;
+          for (int k = 0; k < D / 32; ++k) n2 = fmaf(c[u][k], c[u][k], n2);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+          bool nz = false;
+#pragma unroll
+          for (int k = 0; k < D / 32; ++k) nz |= c[u][k] != 0.f;
+          const bool ok = ((counted >> (b & 31)) & 1u) && b < nb && __any_sync(0xffffffffu, nz);
+          if (ok) {
+            valid |= 1u << b;
+            cmax = fmaxf(cmax, n2);
+            extreme |= !(n2 > 1e-30f && n2 < 1e30f);
+          }
+          const float inv = ok ? rsqrtf(n2) : 0.f;
+#pragma unroll
+          for (int k = 0; k < D / 32; ++k) {
+            const int col = lane + 32 * k;
+            const float x = c[u][k] * inv;
+            const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+            const __nv_bfloat16 lo = __float2bfloat16_rn(x - __bfloat162float(hi));
+            *reinterpret_cast<__nv_bfloat16*>(bm + sw128_offset(b, col, bbox)) = hi;
+            *reinterpret_cast<__nv_bfloat16*>(bm + sw128_offset(nbp + b, col, bbox)) = lo;
+          }
         }
-        if (lane == 0 && b < nb) {
-          bvalid[pb][b] = ok;
-          bool plain = true;
-          DF inv_df{0.f, 0.f};
-          if (ok) inv_df = centroid_inv_norm(n2d, n2, plain);
-          cninv[pb][b] = inv_df;
-          if (!plain) degenerate[pb] = 1;
-        }
+      }
+      if (lane == 0) {
+        kv_sh[wk] = valid;
+        km_sh[wk] = (__float_as_uint(cmax) & 0x7fffffffu) | (extreme ? 0x80000000u : 0u);
       }
       fence_proxy_async_smem();  // generic-proxy writes, read next by the tensor cores
-      named_barrier(3, 32 * kKeepers);
-      if (tk == 0) mbar_arrive(&bready[pb]);
-    };
-    auto fold = [&](int idx) {
-      const int pb = idx & 1;
-      const int e = inst(idx);
-      long long* acc_i = acc + pb * cells;
-      mbar_wait(&accdone[pb], (idx >> 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
-      mbar_wait(&sbar, idx & 1, abort_flag, a.err, kDevTimeoutEpilogue);
-      if (tk < nb) rcp_sh[tk] = count_reciprocal(cnt_old[pb][tk] + add_cnt[pb][tk]);
-      named_barrier(3, 32 * kKeepers);
-      for (int c = tk; c < cells; c += 32 * kKeepers) {
-        const int b = c / D, col = c - b * D;
-        const int ai = b * D + (col % kCols) * 32 + col / kCols;  // the accumulator cell of (b, col)
-        if (add_cnt[pb][b] > 0) {
-          const size_t gi = static_cast<size_t>(e) * cells + c;
-          const double s_new = fold_sum_fp64(sums_sm[c], acc_i[ai]);
-          a.sums[gi] = s_new;
-          a.cent[gi] = centroid_value(s_new, rcp_sh[b]);
+      named_barrier(2, 128);
+      if (wk == 0 && lane == 0) {
+        uint32_t v = 0u, m = 0u, x = 0u;
+        for (int w = 0; w < 4; ++w) {
+          v |= kv_sh[w];
+          m = max(m, km_sh[w] & 0x7fffffffu);
+          x |= km_sh[w] >> 31;
         }
-        acc_i[ai] = 0;  // the cell this thread read: no other thread touches it
+        // |q| < 2^E for what has been seen; before that four times the largest centroid
+        const uint32_t seen = *reinterpret_cast<volatile uint32_t*>(&seen_sh);
+        int E = seen ? ((static_cast<int>(seen >> 23) - 127) >> 1) + 1 : ((static_cast<int>(m >> 23) - 127) >> 1) + 3;
+        E = E < kMinE ? kMinE : E > kMaxE ? kMaxE : E;
+        vmask_sh[slot] = v;
+        exp_sh[slot] = (E & 0xff) | (x ? 0x100 : 0);
+        mbar_arrive(&bready[pb]);
       }
-      named_barrier(3, 32 * kKeepers);
-      if (tk < nb) {
-        if (add_cnt[pb][tk] > 0) a.counts[static_cast<size_t>(e) * nb + tk] = cnt_old[pb][tk] + add_cnt[pb][tk];
-        add_cnt[pb][tk] = 0;
-      }
-      named_barrier(3, 32 * kKeepers);
-      if (tk == 0) {
-        mbar_arrive(&accclear[pb]);
-        if (idx + 1 < n_my) issue_sums(idx + 1);
-        if (idx + 2 < n_my) issue_cent(idx + 2);
-      }
-    };
-
-    if (n_my > 0) {
-      if (tk == 0) {
-        issue_cent(0);
-        issue_sums(0);
-        if (n_my > 1) issue_cent(1);
-      }
-      build(0);
-      for (int i = 0; i < n_my; ++i) {
-        if (i + 1 < n_my) build(i + 1);
-        fold(i);
-      }
+      named_barrier(2, 128);  // kv_sh and km_sh are free again
     }
   }
 
@@ -665,10 +924,33 @@ __global__ void __launch_bounds__(kUThreads, 1)
   }
 }
 
+template <int D, int NBO>
+cudaError_t launch_update_dn(const UpdArgs& a, const CUtensorMap& qmap, int grid, cudaStream_t st) {
+  using C = UpdCfg<D, NBO>;
+  const size_t smem = C::smem_bytes(a.nbp);
+  const cudaError_t e =
+      cudaFuncSetAttribute(update_kernel<D, NBO>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  update_kernel<D, NBO><<<grid, kUThreads, smem, st>>>(qmap, a, C::stages(a.nbp));
+  return cudaGetLastError();
+}
+
+int update_grid(int n_inst) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return n_inst < sms ? n_inst : sms;
+}
+
 }  // namespace
 
-cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows, int n_new, float* cent,
-                          double* sums, long long* counts, int* assign_out, int* err, cudaStream_t st) {
+size_t update_spill_words(const Shape& s) {
+  return s.nb == 0 ? 0 : static_cast<size_t>(update_grid(s.n_inst)) * kSpillSlots * s.nb * s.d;
+}
+
+cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows, int n_new,
+                          float* cent, double* sums, long long* counts, int* assign_out, unsigned long long* spill,
+                          int* err, cudaStream_t st) {
   UpdArgs a;
   a.n_inst = s.n_inst;
   a.nq = s.G * n_new;
@@ -679,27 +961,12 @@ cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows,
   a.sums = sums;
   a.counts = counts;
   a.assign_out = assign_out;
+  a.spill = spill;
   a.err = err;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int grid = s.n_inst < sms ? s.n_inst : sms;
-  if (s.d == 128) {
-    using C = UpdCfg<128>;
-    const size_t smem = C::smem_bytes(a.nb, a.nbp);
-    cudaError_t e =
-        cudaFuncSetAttribute(update_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    update_kernel<128><<<grid, kUThreads, smem, st>>>(qmap, a, C::stages(a.nb, a.nbp));
-  } else {
-    using C = UpdCfg<64>;
-    const size_t smem = C::smem_bytes(a.nb, a.nbp);
-    cudaError_t e =
-        cudaFuncSetAttribute(update_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    update_kernel<64><<<grid, kUThreads, smem, st>>>(qmap, a, C::stages(a.nb, a.nbp));
-  }
-  return cudaGetLastError();
+  const int grid = update_grid(s.n_inst);
+  if (s.d == 128)
+    return s.nb <= 16 ? launch_update_dn<128, 16>(a, qmap, grid, st) : launch_update_dn<128, 32>(a, qmap, grid, st);
+  return s.nb <= 16 ? launch_update_dn<64, 16>(a, qmap, grid, st) : launch_update_dn<64, 32>(a, qmap, grid, st);
 }
 
 }  // namespace bkv

@@ -294,6 +294,50 @@ __device__ __forceinline__ float centroid_value(double s, DF rcp) {
   return __fadd_rn(p, err);
 }
 
+// The common case of fold_sum and centroid_value at once, in 32-bit integer steps and without a branch
+// (several cells' latencies overlap): s a multiple of 2^-40 below 2^22, |acc| < 2^61 and a nonzero total
+// t = s * 2^40 + acc.  Returns false, with meaningless outputs, otherwise.  t's leading bit p is shifted
+// to bit 63; its top 53 bits, rounded to nearest even, are the double's significand, whose own
+// rounding to 24 bits and remainder are centroid_value's hi = m_hi * 2^(p - 63) and lo = rem * 2^(p - 92).
+__device__ __forceinline__ bool fold_and_centroid(double s, long long acc, DF rcp, double& s_new, float& c_new) {
+  const uint32_t shi = static_cast<uint32_t>(__double2hiint(s)), slo = static_cast<uint32_t>(__double2loint(s));
+  const int sh = 1035 - static_cast<int>((shi >> 20) & 0x7ffu);  // s * 2^40 = significand / 2^sh
+  const unsigned long long sm = (static_cast<unsigned long long>((shi & 0xfffffu) | 0x100000u) << 32) | slo;
+  const bool zero = ((shi << 1) | slo) == 0u;
+  const unsigned long long sv = sh >= 0 ? sm >> (sh & 63) : sm << (-sh & 63);
+  bool ok = zero || (sh > -10 && sh < 53 && (sh < 0 || (sv << (sh & 63)) == sm));
+  const long long f = zero ? 0ll : (shi >> 31) ? -static_cast<long long>(sv) : static_cast<long long>(sv);
+  const long long t = f + acc;
+  ok = ok && t != 0 && acc > -(1ll << 61) && acc < (1ll << 61);
+  const unsigned long long a = static_cast<unsigned long long>(t < 0 ? -t : t);
+  const int lz = __clzll(static_cast<long long>(a | 1ull));
+  const unsigned long long n = a << lz;
+  unsigned long long m = n >> 11;
+  const uint32_t low = static_cast<uint32_t>(n) & 0x7ffu;
+  m += low + (static_cast<uint32_t>(m) & 1u) > 0x400u ? 1u : 0u;
+  const int carry = static_cast<int>(m >> 53);  // 1: rounded up to a power of two
+  const int p = 63 - lz + carry;
+  m >>= carry;
+  const uint32_t mhi = static_cast<uint32_t>(m >> 32), mlo = static_cast<uint32_t>(m);
+  const uint32_t sign = t < 0 ? 0x80000000u : 0u;
+  s_new = __hiloint2double(static_cast<int>(sign | (static_cast<uint32_t>(p + 983) << 20) | (mhi & 0xfffffu)),
+                           static_cast<int>(mlo));
+  const uint32_t top = __funnelshift_l(mlo, mhi, 3);  // m >> 29: 24 bits
+  const int r = static_cast<int>(mlo & 0x1fffffffu);
+  const int up = r + static_cast<int>(top & 1u) > 0x10000000 ? 1 : 0;  // to nearest, ties to even
+  const int rem = r - (up << 29);
+  const float mh = __int_as_float(static_cast<int>(top) + up + 0x4A800000);
+  const float rem_f = __fadd_rn(__fmul_rn(magic_i2f(rem >> 6), 64.f), magic_i2f(rem & 63));
+  const float hi = __uint_as_float(__float_as_uint(__fmul_rn(mh, pow2f(p - 63))) | sign);
+  const float lo = __uint_as_float(__float_as_uint(__fmul_rn(rem_f, pow2f(p - 92))) ^ sign);
+  const float q = __fmul_rn(hi, rcp.hi);
+  float err = __fmaf_rn(hi, rcp.hi, -q);
+  err = __fmaf_rn(hi, rcp.lo, err);
+  err = __fmaf_rn(lo, rcp.hi, err);
+  c_new = __fadd_rn(q, err);
+  return ok;
+}
+
 // Exact assignment of one query (warp-wide; x holds this lane's elements lane + 32 j):
 // the valid beacon maximising (q . c_b) * (1 / |c_b|) in double-float arithmetic (exact
 // products, TwoSum accumulation, then a butterfly over the lanes), ties to the lower
