@@ -38,6 +38,12 @@
 // quarter: in pass 1 each owns half of the query columns, in pass 2 each
 // takes every other tile with all columns.
 //
+// TMA and MMAs are issued under elect.sync, which keeps their operands in uniform
+// registers (see elect_one): the eight MMAs of a tile then take their own time,
+// about 530 clocks, instead of 760 of issue.  4608 instances of 4224 keys, 48
+// queries: 922 -> 906 us (733 at the copy rate); 2560 of 8320, 56 queries: 1313 ->
+// 1278 us (802).
+//
 // Cross-CTA exchange (all waits bounded): barriers are initialised, then a
 // cluster barrier.  Per instance every CTA pushes its (m, s) column partials
 // into each peer's receive buffer with st.async, whose bytes complete on the
@@ -451,7 +457,7 @@ __global__ void __launch_bounds__(kScThreads, 1)
   // pass-1 jobs for tiles 0 .. T-1, then pass-2 jobs for the streaming tiles.
   if (warp == 0) {
     // ---------------------------------------------------------------- producer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint64_t once = l2_policy_evict_first(), again = l2_policy_evict_last();
       prefetch_tmap(&kmap);
       prefetch_tmap(&kmap32);
@@ -508,7 +514,7 @@ __global__ void __launch_bounds__(kScThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = idesc_bf16_f32(128, N);
       int g = 0, ks = 0, kp2_0 = 0, kp2_1 = 0;  // pass-1 streaming uses; pass-2 uses per half
       int rs = 0, ru = 0;                        // next ring slot and its use count
