@@ -35,11 +35,9 @@
  * Streams.  All work is enqueued on the CUDA stream given to bkv_create (or
  * bkv_set_stream); calls return before it completes.  Outputs are valid once
  * that stream has been synchronised (bkv_sync does so and reports device-side
- * errors).  bkv_compress stages its rotary table in one of four pinned host
- * buffers, which a kernel on the stream copies to the device (no copy-engine
- * transfer, so the stream does not queue behind other streams' bulk host
- * copies), and waits only when the stream is more than four compress calls
- * behind.  One context must not be used from two host threads at once.
+ * errors).  A compress passes its positions in kernel parameters and computes
+ * its rotary table on the device: no call copies from host memory or waits for
+ * the stream.  One context must not be used from two host threads at once.
  *
  * Errors.  Every call returns BKV_OK (0) or a negative code; nothing throws.
  * Argument errors are detected on the host before any work is enqueued and
@@ -332,7 +330,7 @@ int bkv_selftest_bounds(bkv_ctx* ctx);
 
 /*
  * Allocation-failure hook (test diagnostic).  With nth > 0, the nth device
- * or pinned host allocation that later bkv_create calls attempt (counted
+ * allocation that later bkv_create calls attempt (counted
  * from this call, across contexts) fails as if memory ran out, without
  * allocating: that bkv_create releases what it had allocated, leaves *out
  * NULL and returns BKV_ENOMEM.  The hook disarms itself after that one
@@ -356,7 +354,7 @@ int bkv_debug_fail_alloc(int32_t nth);
 #define BKV_K_SELECT_GATHER 4
 #define BKV_K_KEEP_ALL 5
 #define BKV_K_CFPS 6 /* Continual FPS buffer update, beacon selection and merge */
-#define BKV_K_ROPE 7 /* rotary table of a compress, copied from pinned host memory */
+#define BKV_K_ROPE 7 /* rotary tables (and causal gaps) of a compress */
 #define BKV_NUM_KERNELS 8
 int bkv_profile_enable(bkv_ctx* ctx, int on);
 int bkv_profile_read(bkv_ctx* ctx, double* ms, int64_t* launches, int32_t n_kernels);
@@ -385,9 +383,9 @@ int bkv_profile_read(bkv_ctx* ctx, double* ms, int64_t* launches, int32_t n_kern
  *               kernel's bounded wait expires or, in a checked build, a
  *               device-side bounds check fails (outputs are then invalid).
  *   err_msg     host buffer of err_len bytes or NULL: reason of a failure.
- * The rotary table (rope_theta != 0) reaches the device inside the
- * parameters of small kernels on `stream`, 16 KB per launch: no copy from
- * host memory, and the call does not wait for earlier work on the stream.
+ * The rotary table (rope_theta != 0) is computed on the device from the
+ * positions, passed in the parameters of a small kernel on `stream`: no copy
+ * from host memory, and the call does not wait for earlier work on the stream.
  * All calls share the scratch array and it keeps the previous call's
  * contents; calls that overlap on the GPU (other streams, other threads
  * without ordering) race on it.  The array's device address is looked up

@@ -41,26 +41,13 @@ struct bkv_ctx {
   float* rscore = nullptr;        // [n_inst][cap]
   double2* rope = nullptr;        // [W + 1][d / 2] fp64 (cos, sin), then the same table in fp32
   int* err = nullptr;             // device error word
-  // pinned host staging of the rotary table, a ring of kRopeSlots: a compress fills the next slot,
-  // a kernel on the stream copies it to `rope` through the slot's device mapping, and the slot is
-  // refilled only after that copy's event completed
-  static constexpr int kRopeSlots = 4;
-  double2* rope_pinned[kRopeSlots] = {};
-  void* rope_mapped[kRopeSlots] = {};  // device address of rope_pinned[i]
-  cudaEvent_t rope_ev[kRopeSlots] = {};
-  bool rope_used[kRopeSlots] = {};
-  int rope_next = 0;
+  double inv_freq[64] = {};       // theta^(-2i / d), i < d / 2
   // per-instance lengths (bkv_compress_ragged): the instances a compress evicts from, and a rotary
-  // table per batch row followed by the causal gaps [batch][W] (int32), staged like `rope`
+  // table per batch row followed by the causal gaps [batch][W] (int32)
   int* work = nullptr;            // [n_inst]
   int* n_work = nullptr;          // [1]
-  unsigned char* rag = nullptr;   // device copy of the per-row tables and gaps
+  unsigned char* rag = nullptr;
   size_t rag_bytes = 0, rag_row = 0, rag_gaps_off = 0;  // total bytes; one row's table (double2 units); gaps offset
-  void* rag_pinned[kRopeSlots] = {};
-  void* rag_mapped[kRopeSlots] = {};
-  cudaEvent_t rag_ev[kRopeSlots] = {};
-  bool rag_used[kRopeSlots] = {};
-  int rag_next = 0;
   cudaEvent_t switch_ev = nullptr;  // orders a new stream after the previous one (bkv_set_stream)
   std::string last_error;
   // per-kernel timing
@@ -178,8 +165,8 @@ int validate_config(const bkv_config* cfg, std::string& why) {
   return BKV_OK;
 }
 
-// Allocation-failure hook (bkv_debug_fail_alloc): once armed with n > 0, the n-th device or pinned
-// host allocation that bkv_create attempts reports cudaErrorMemoryAllocation without allocating,
+// Allocation-failure hook (bkv_debug_fail_alloc): once armed with n > 0, the n-th device
+// allocation that bkv_create attempts reports cudaErrorMemoryAllocation without allocating,
 // and the hook disarms itself.
 std::atomic<int> g_fail_nth{0};
 std::atomic<int> g_alloc_seen{0};
@@ -195,12 +182,6 @@ template <typename T>
 cudaError_t dmalloc(T** p, size_t n) {
   if (fail_this_alloc()) return cudaErrorMemoryAllocation;
   return cudaMalloc(reinterpret_cast<void**>(p), sizeof(T) * (n ? n : 1));
-}
-
-template <typename T>
-cudaError_t hmalloc(T** p, size_t bytes) {
-  if (fail_this_alloc()) return cudaErrorMemoryAllocation;
-  return cudaMallocHost(reinterpret_cast<void**>(p), bytes);
 }
 
 void free_all(bkv_ctx* c) {
@@ -222,12 +203,6 @@ void free_all(bkv_ctx* c) {
   cudaFree(c->rscore);
   cudaFree(c->rope);
   cudaFree(c->err);
-  for (int i = 0; i < bkv_ctx::kRopeSlots; ++i) {
-    if (c->rope_pinned[i]) cudaFreeHost(c->rope_pinned[i]);
-    if (c->rope_ev[i]) cudaEventDestroy(c->rope_ev[i]);
-    if (c->rag_pinned[i]) cudaFreeHost(c->rag_pinned[i]);
-    if (c->rag_ev[i]) cudaEventDestroy(c->rag_ev[i]);
-  }
   cudaFree(c->work);
   cudaFree(c->n_work);
   cudaFree(c->rag);
@@ -291,6 +266,7 @@ int bkv_create(const bkv_config* cfg, void* stream, bkv_ctx** out) {
   c->rag_row = static_cast<size_t>(s.W + 1) * (s.d / 2) * 3 / 2;  // double2 units (a multiple of 2: 16-byte rows)
   c->rag_gaps_off = sizeof(double2) * c->rag_row * static_cast<size_t>(s.batch);
   c->rag_bytes = c->rag_gaps_off + (sizeof(int32_t) * static_cast<size_t>(s.batch) * (s.W > 0 ? s.W : 1) + 15) / 16 * 16;
+  bkv::rope_frequencies(cfg->rope_theta, s.d, c->inv_freq);
   cudaGetDevice(&c->device);
 
   const size_t ni = static_cast<size_t>(s.n_inst);
@@ -325,21 +301,6 @@ int bkv_create(const bkv_config* cfg, void* stream, bkv_ctx** out) {
     free_all(c);
     delete c;
     return BKV_ECUDA;
-  }
-  const size_t rope_bytes = sizeof(double2) * (static_cast<size_t>(s.W + 1) * (s.d / 2) * 3 / 2 + 1);
-  for (int i = 0; i < bkv_ctx::kRopeSlots; ++i) {
-    if ((e = hmalloc(&c->rope_pinned[i], rope_bytes)) != cudaSuccess ||
-        (e = cudaHostGetDevicePointer(&c->rope_mapped[i], c->rope_pinned[i], 0)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&c->rope_ev[i], cudaEventDisableTiming)) != cudaSuccess ||
-        (e = hmalloc(&c->rag_pinned[i], c->rag_bytes)) != cudaSuccess ||
-        (e = cudaHostGetDevicePointer(&c->rag_mapped[i], c->rag_pinned[i], 0)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&c->rag_ev[i], cudaEventDisableTiming)) != cudaSuccess) {
-      const int code = (e == cudaErrorMemoryAllocation) ? BKV_ENOMEM : BKV_ECUDA;
-      cudaGetLastError();
-      free_all(c);
-      delete c;
-      return code;
-    }
   }
   if ((e = cudaEventCreateWithFlags(&c->switch_ev, cudaEventDisableTiming)) != cudaSuccess) {
     cudaGetLastError();
@@ -523,35 +484,12 @@ int bkv_compress(bkv_ctx* ctx, void* K, void* V, int32_t L, int32_t budget, int6
   if (s.nb > 0 && !ctx->state_ready) return fail(ctx, BKV_ESTATE, "compress before bkv_init_beacons / bkv_set_state");
 
   // rotary table: slot w < W is recent_pos[w], slot W is t_pos
-  const int h = s.d / 2;
-  const double theta = ctx->cfg.rope_theta;
-  const int rotate = theta != 0.0;
+  const int rotate = ctx->cfg.rope_theta != 0.0;
   if (rotate) {
-    const size_t n = static_cast<size_t>(s.W + 1) * h;
-    const int rs = ctx->rope_next;
-    ctx->rope_next = (rs + 1) % bkv_ctx::kRopeSlots;
-    if (ctx->rope_used[rs] && (e = cudaEventSynchronize(ctx->rope_ev[rs])) != cudaSuccess)
-      return cuda_fail(ctx, e, "rope staging wait");
-    double2* tab = ctx->rope_pinned[rs];
-    float2* tab32 = reinterpret_cast<float2*>(tab + n);
-    for (int slot = 0; slot <= s.W; ++slot) {
-      const double pos = static_cast<double>(slot < s.W ? recent_pos[slot] : t_pos);
-      for (int i = 0; i < h; ++i) {
-        const double inv_freq = std::pow(theta, -static_cast<double>(2 * i) / static_cast<double>(s.d));
-        const double ang = pos * inv_freq;
-        const double c = std::cos(ang), sn = std::sin(ang);
-        tab[static_cast<size_t>(slot) * h + i] = make_double2(c, sn);
-        tab32[static_cast<size_t>(slot) * h + i] = make_float2(static_cast<float>(c), static_cast<float>(sn));
-      }
-    }
-    {  // the slot is not refilled before this copy's event
-      ProfScope ps(ctx, BKV_K_ROPE);
-      e = bkv::launch_rope_stage(ctx->rope_mapped[rs], ctx->rope, sizeof(double2) * n + sizeof(float2) * n,
-                                 ctx->stream);
-    }
-    if (e == cudaSuccess) e = cudaEventRecord(ctx->rope_ev[rs], ctx->stream);
-    ctx->rope_used[rs] = true;
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "rope table upload");
+    ProfScope ps(ctx, BKV_K_ROPE);
+    e = bkv::launch_rope_table(s.W, s.d / 2, 1, ctx->inv_freq, &t_pos, recent_pos, 1, ctx->rope, 0, nullptr, 0,
+                               ctx->stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "rope table launch");
   }
   bkv::CfpsArgs ca{};
   if (ctx->cfps) {  // this compress's beacons: FPS of each head's buffer, into cent / counts
@@ -647,43 +585,15 @@ int bkv_compress_ragged(bkv_ctx* ctx, void* K, void* V, const int32_t* L, int32_
 
   // per batch row: the rotary table (slot w < W at recent_pos[b][w], slot W at t_pos[b]), then the
   // causal gaps t_pos[b] - recent_pos[b][w], clamped to [0, capacity + 1]
-  const int h = s.d / 2;
-  const double theta = ctx->cfg.rope_theta;
-  const int rotate = theta != 0.0;
-  {
-    const int rs = ctx->rag_next;
-    ctx->rag_next = (rs + 1) % bkv_ctx::kRopeSlots;
-    if (ctx->rag_used[rs] && (e = cudaEventSynchronize(ctx->rag_ev[rs])) != cudaSuccess)
-      return cuda_fail(ctx, e, "ragged staging wait");
-    unsigned char* host = static_cast<unsigned char*>(ctx->rag_pinned[rs]);
-    const size_t n = static_cast<size_t>(s.W + 1) * h;
-    for (int b = 0; b < s.batch; ++b) {
-      double2* tab = reinterpret_cast<double2*>(host) + static_cast<size_t>(b) * ctx->rag_row;
-      float2* tab32 = reinterpret_cast<float2*>(tab + n);
-      for (int slot = 0; rotate && slot <= s.W; ++slot) {
-        const double pos = static_cast<double>(slot < s.W ? recent_pos[static_cast<size_t>(b) * s.W + slot] : t_pos[b]);
-        for (int i = 0; i < h; ++i) {
-          const double inv_freq = std::pow(theta, -static_cast<double>(2 * i) / static_cast<double>(s.d));
-          const double ang = pos * inv_freq;
-          const double c = std::cos(ang), sn = std::sin(ang);
-          tab[static_cast<size_t>(slot) * h + i] = make_double2(c, sn);
-          tab32[static_cast<size_t>(slot) * h + i] = make_float2(static_cast<float>(c), static_cast<float>(sn));
-        }
-      }
-      int32_t* gaps = reinterpret_cast<int32_t*>(host + ctx->rag_gaps_off) + static_cast<size_t>(b) * s.W;
-      for (int w = 0; w < s.W; ++w) {
-        const int64_t rp = recent_pos[static_cast<size_t>(b) * s.W + w];
-        const int64_t g = rp >= t_pos[b] ? 0 : static_cast<int64_t>(static_cast<uint64_t>(t_pos[b]) - static_cast<uint64_t>(rp));
-        gaps[w] = static_cast<int32_t>(g > s.cap + 1LL || g < 0 ? s.cap + 1LL : g);
-      }
-    }
-    {
-      ProfScope ps(ctx, BKV_K_ROPE);
-      e = bkv::launch_rope_stage(ctx->rag_mapped[rs], ctx->rag, ctx->rag_bytes, ctx->stream);
-    }
-    if (e == cudaSuccess) e = cudaEventRecord(ctx->rag_ev[rs], ctx->stream);
-    ctx->rag_used[rs] = true;
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "ragged table upload");
+  const int rotate = ctx->cfg.rope_theta != 0.0;
+  const bool causal = (ctx->cfg.flags & BKV_F_CAUSAL_WINDOW) != 0 && s.W > 0;
+  if (rotate || causal) {
+    ProfScope ps(ctx, BKV_K_ROPE);
+    e = bkv::launch_rope_table(s.W, s.d / 2, s.batch, ctx->inv_freq, t_pos, recent_pos, rotate,
+                               reinterpret_cast<double2*>(ctx->rag), ctx->rag_row,
+                               causal ? reinterpret_cast<int*>(ctx->rag + ctx->rag_gaps_off) : nullptr, s.cap + 1,
+                               ctx->stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "ragged table launch");
   }
   {
     ProfScope ps(ctx, BKV_K_KEEP_ALL);
@@ -724,7 +634,7 @@ int bkv_compress_ragged(bkv_ctx* ctx, void* K, void* V, const int32_t* L, int32_
   sa.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(s.d)));
   sa.valid = ctx->valid;
   sa.mean = (ctx->cfg.flags & BKV_F_MEAN_AGG) != 0;
-  sa.causal = (ctx->cfg.flags & BKV_F_CAUSAL_WINDOW) != 0 && s.W > 0;
+  sa.causal = causal;
   sa.r_out = ctx->rscore;
   sa.err = ctx->err;
   sa.Ls = L;

@@ -81,9 +81,14 @@ cudaError_t launch_update_seq(const Shape& s, const __nv_bfloat16* q_steps, int 
 // rope: [W + 1][d / 2] fp64 (cos, sin) pairs, immediately followed by the same
 // [W + 1][d / 2] table as fp32 pairs; entry w < W is recent slot w, entry W
 // is the beacon position.  rotate == 0 leaves vectors unrotated.
-// Device copy of `bytes` (a multiple of 16, both ends 16-byte aligned) from a
-// device-mapped pinned host buffer, by a kernel on `st`.
-cudaError_t launch_rope_stage(const void* src, void* dst, size_t bytes, cudaStream_t st);
+// launch_rope_table writes the tables of `rows` batch rows (row b at table + b * row_stride, double2 units)
+// from host positions: t_pos[rows] and recent_pos[rows][W], passed by value in kernel parameters.
+// inv_freq [d / 2] (host): theta^(-2i / d).  gaps (device [rows][W] or nullptr): t_pos - recent_pos of each
+// slot clamped to [0, gap_max], 0 at or after t_pos.  rotate == 0 writes the gaps only.
+cudaError_t launch_rope_table(int W, int h, int rows, const double* inv_freq, const int64_t* t_pos,
+                              const int64_t* recent_pos, int rotate, double2* table, size_t row_stride, int* gaps,
+                              int gap_max, cudaStream_t st);
+void rope_frequencies(double theta, int d, double* inv_freq);
 cudaError_t launch_qobs(const Shape& s, const __nv_bfloat16* q_recent, const float* cent, const long long* counts,
                         const double2* rope, int rotate, __nv_bfloat16* qobs, uint32_t* valid, int* err,
                         cudaStream_t st);

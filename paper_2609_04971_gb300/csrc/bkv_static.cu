@@ -23,10 +23,9 @@
 //     the first time this entry point runs on a device (with that device
 //     current), so that first call should come before any stream capture.
 //
-// The rotary table of a call (at most 65 positions x 64 frequency pairs, in
-// fp64 and fp32) reaches the device as by-value kernel parameters, in chunks
-// of 16 KB that a small kernel writes into the array: no copy from pageable
-// host memory, so the call never waits for the stream.
+// The rotary table of a call is computed on the device from at most 65 positions
+// and 64 frequencies passed as kernel parameters: no copy from host memory, so
+// the call never waits for the stream.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -78,53 +77,6 @@ bool encode(CUtensorMap* map, const void* base, uint64_t rows, int d, uint32_t b
 }
 
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
-
-// One chunk of the rotary table, passed by value: 16-byte units [first, first + count).
-constexpr int kRopeChunkUnits = 1024;
-struct RopeChunk {
-  uint32_t first, count;
-  uint4 unit[kRopeChunkUnits];
-};
-
-__global__ void __launch_bounds__(256) rope_param_kernel(const __grid_constant__ RopeChunk c, uint4* table) {
-  for (uint32_t i = threadIdx.x; i < c.count; i += blockDim.x) table[c.first + i] = c.unit[i];
-}
-
-// 16-byte unit u of the table laid out as bkv_compress lays it out: units [0, n) are the fp64
-// (cos, sin) entries, units [n, 3n/2) two fp32 (cos, sin) entries each (n is even: d/2 is 32 or 64).
-// Entry k is slot k / h (recent slot w < W at recent_pos[w], slot W at t_pos), frequency k % h.
-struct RopeTable {
-  double theta;
-  int d, h, W;
-  int64_t t_pos;
-  const int64_t* recent_pos;
-  size_t n;
-  void entry(size_t k, double& c, double& s) const {
-    const int slot = static_cast<int>(k / h), i = static_cast<int>(k % h);
-    const double pos = static_cast<double>(slot < W ? recent_pos[slot] : t_pos);
-    const double inv_freq = std::pow(theta, -static_cast<double>(2 * i) / static_cast<double>(d));
-    const double ang = pos * inv_freq;
-    c = std::cos(ang);
-    s = std::sin(ang);
-  }
-  uint4 unit(size_t u) const {
-    uint4 out;
-    double c, s;
-    if (u < n) {
-      entry(u, c, s);
-      const double2 v = make_double2(c, s);
-      std::memcpy(&out, &v, sizeof out);
-    } else {
-      float2 v[2];
-      for (int j = 0; j < 2; ++j) {
-        entry(2 * (u - n) + j, c, s);
-        v[j] = make_float2(static_cast<float>(c), static_cast<float>(s));
-      }
-      std::memcpy(&out, v, sizeof out);
-    }
-    return out;
-  }
-};
 
 }  // namespace
 
@@ -215,23 +167,14 @@ extern "C" int bkv_compress_static(const bkv_config* cfg, const float* centroids
   auto* rscore = reinterpret_cast<float*>(b + off_score);
   auto* rope = reinterpret_cast<double2*>(b + off_rope);
 
-  const int h = s.d / 2;
-  const double theta = cfg->rope_theta;
-  const int rotate = theta != 0.0;
+  const int rotate = cfg->rope_theta != 0.0;
   if (rotate) {
-    // fp64 (cos, sin) entries followed by the same entries in fp32, as kernel parameters
-    const RopeTable tab{theta, s.d, h, s.W, t_pos, recent_pos, static_cast<size_t>(s.W + 1) * h};
-    const size_t units = tab.n + tab.n / 2;
-    RopeChunk chunk;
-    for (size_t u0 = 0; u0 < units; u0 += kRopeChunkUnits) {
-      chunk.first = static_cast<uint32_t>(u0);
-      chunk.count = static_cast<uint32_t>(std::min<size_t>(kRopeChunkUnits, units - u0));
-      for (uint32_t i = 0; i < chunk.count; ++i) chunk.unit[i] = tab.unit(u0 + i);
-      rope_param_kernel<<<1, 256, 0, st>>>(chunk, reinterpret_cast<uint4*>(rope));
-      if ((e = cudaGetLastError()) != cudaSuccess) {
-        message(err_msg, err_len, cudaGetErrorString(e));
-        return BKV_ECUDA;
-      }
+    double inv_freq[64];
+    bkv::rope_frequencies(cfg->rope_theta, s.d, inv_freq);
+    e = bkv::launch_rope_table(s.W, s.d / 2, 1, inv_freq, &t_pos, recent_pos, 1, rope, 0, nullptr, 0, st);
+    if (e != cudaSuccess) {
+      message(err_msg, err_len, cudaGetErrorString(e));
+      return BKV_ECUDA;
     }
   }
   e = bkv::launch_qobs(s, static_cast<const __nv_bfloat16*>(q_recent), centroids,

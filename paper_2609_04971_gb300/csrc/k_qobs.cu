@@ -9,7 +9,7 @@
 //
 // Definition of each output element: y_i = x_i c - x_{i+d/2} s and
 // y_{i+d/2} = x_{i+d/2} c + x_i s evaluated in fp64 (separately rounded
-// products, host-computed fp64 cos / sin), then rounded fp64 -> fp32 -> bf16.
+// products, fp64 cos / sin), then rounded fp64 -> fp32 -> bf16.
 // The kernel first evaluates y in fp32 (one FMA, fp32 copies of cos / sin).
 // The fp32 value v differs from the fp64 one by at most
 //   delta = 2^-22 (|x_a| + |x_b| + |v|)
@@ -19,6 +19,8 @@
 // one fp32 ulp of it; if v is farther than delta + 1 ulp from the nearest
 // midpoint, bf16(v) is the defined value.  Otherwise (about 2e-4 of the
 // elements) the element is recomputed in fp64 exactly as defined.
+#include <cmath>
+
 #include "bkv_device.cuh"
 #include "bkv_internal.h"
 
@@ -120,25 +122,76 @@ __global__ void __launch_bounds__(kQobsThreads) qobs_kernel(Shape s, const __nv_
   }
 }
 
-// Copies one compress's rotary table from pinned host memory, read through its
-// device mapping, into device memory.  The copy is made by the SMs rather than
-// a copy engine, so the stream's kernels never wait in a copy-engine queue
-// behind bulk host transfers that other streams have issued.
-__global__ void __launch_bounds__(256) rope_stage_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
-                                                         int n16) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n16) dst[i] = src[i];
+// One chunk of positions, by value: rows of W + 1 positions (the recent slots, then t_pos).
+constexpr int kRopePositions = 1024;
+template <int N>
+struct RopeChunk {
+  double inv_freq[64];
+  long long pos[N];
+};
+
+// Rotary tables (and causal gaps) of a chunk of batch rows: block = one position, thread = one frequency
+// pair.  The angle is the fp64 product of position and frequency, its cosine and sine are CUDA's fp64
+// ones (within 2 ulp, far below what the fp64 -> fp32 -> bf16 rounding of a rotated query can see).
+// Formed on the host (576 pow, cos and sin for 8 recent slots and d = 128) the table cost a compress about
+// 50 us of host time before its first launch, and a copy kernel reading pinned memory.
+template <int N>
+__global__ void __launch_bounds__(64) rope_table_kernel(const __grid_constant__ RopeChunk<N> c, int first_row, int W,
+                                                        int h, int rotate, double2* table, size_t row_stride, int* gaps,
+                                                        int gap_max) {
+  const int row = blockIdx.x / (W + 1), slot = blockIdx.x % (W + 1), i = threadIdx.x;
+  const long long pos = c.pos[blockIdx.x];
+  if (rotate) {
+    double2* tab = table + static_cast<size_t>(first_row + row) * row_stride;
+    float2* tab32 = reinterpret_cast<float2*>(tab + static_cast<size_t>(W + 1) * h);
+    double sn, cs;
+    sincos(__dmul_rn(static_cast<double>(pos), c.inv_freq[i]), &sn, &cs);
+    tab[slot * h + i] = make_double2(cs, sn);
+    tab32[slot * h + i] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
+  }
+  if (gaps && i == 0 && slot < W) {
+    const long long t = c.pos[row * (W + 1) + W];
+    const long long g = pos >= t ? 0 : static_cast<long long>(static_cast<unsigned long long>(t) - static_cast<unsigned long long>(pos));
+    gaps[(first_row + row) * W + slot] = static_cast<int>(g > gap_max || g < 0 ? gap_max : g);
+  }
+}
+
+template <int N>
+cudaError_t launch_rope_chunks(int W, int h, int rows, const double* inv_freq, const int64_t* t_pos,
+                               const int64_t* recent_pos, int rotate, double2* table, size_t row_stride, int* gaps,
+                               int gap_max, cudaStream_t st) {
+  RopeChunk<N> c;
+  for (int i = 0; i < h; ++i) c.inv_freq[i] = inv_freq[i];
+  const int per = N / (W + 1);  // rows per launch (at least one: W <= 64)
+  for (int r0 = 0; r0 < rows; r0 += per) {
+    const int n = rows - r0 < per ? rows - r0 : per;
+    for (int r = 0; r < n; ++r) {
+      long long* pos = c.pos + r * (W + 1);
+      for (int w = 0; w < W; ++w) pos[w] = recent_pos[static_cast<size_t>(r0 + r) * W + w];
+      pos[W] = t_pos[r0 + r];
+    }
+    rope_table_kernel<N><<<n * (W + 1), h, 0, st>>>(c, r0, W, h, rotate, table, row_stride, gaps, gap_max);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace
 
-cudaError_t launch_rope_stage(const void* src, void* dst, size_t bytes, cudaStream_t st) {
-  if (bytes == 0) return cudaSuccess;
-  if (bytes % 16 != 0 || (reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) % 16 != 0)
-    return cudaErrorInvalidValue;
-  const int n16 = static_cast<int>(bytes / 16);
-  rope_stage_kernel<<<(n16 + 255) / 256, 256, 0, st>>>(static_cast<const uint4*>(src), static_cast<uint4*>(dst), n16);
-  return cudaGetLastError();
+void rope_frequencies(double theta, int d, double* inv_freq) {
+  for (int i = 0; i < d / 2; ++i)
+    inv_freq[i] = theta != 0.0 ? std::pow(theta, -static_cast<double>(2 * i) / static_cast<double>(d)) : 0.0;
+}
+
+cudaError_t launch_rope_table(int W, int h, int rows, const double* inv_freq, const int64_t* t_pos,
+                              const int64_t* recent_pos, int rotate, double2* table, size_t row_stride, int* gaps,
+                              int gap_max, cudaStream_t st) {
+  // a single row's parameters stay small (at most 65 positions)
+  return rows == 1 ? launch_rope_chunks<kMaxWindow + 1>(W, h, rows, inv_freq, t_pos, recent_pos, rotate, table,
+                                                        row_stride, gaps, gap_max, st)
+                   : launch_rope_chunks<kRopePositions>(W, h, rows, inv_freq, t_pos, recent_pos, rotate, table,
+                                                        row_stride, gaps, gap_max, st);
 }
 
 cudaError_t launch_qobs(const Shape& s, const __nv_bfloat16* q_recent, const float* cent, const long long* counts,

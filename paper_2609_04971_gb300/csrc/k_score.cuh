@@ -76,6 +76,8 @@
 // form, k_score_mean.cu the mean form and k_score_causal*.cu their causal
 // forms, so that they compile in parallel.
 #pragma once
+#include <mutex>
+
 #include "bkv_device.cuh"
 #include "bkv_internal.h"
 
@@ -870,23 +872,35 @@ cudaError_t launch_score_dq(const Shape& s, const CUtensorMap& kmap, const CUten
                             const CUtensorMap& qmap, const ScoreArgs& a, cudaStream_t st) {
   using C = ScoreCfg<D>;
   auto kern = score_kernel<D, NQ, MEAN, CAUSAL, COMBINE>;
-  int dev = 0, sms = 0, max_clusters = 0;
+  int dev = 0;
   cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // SMs that clusters of each size keep busy, queried once per device for this kernel (the shared
-  // memory of a cluster's CTAs grows with its size by a few bytes only, so the largest is used)
-  static int busy[kMaxDevicesScore][kMaxCluster + 1] = {};
+  // Set up once per device for this kernel: its limits, and the SMs that clusters of each size keep busy
+  // (the shared memory of a cluster's CTAs grows with its size by a few bytes only, so the largest size's
+  // is used).  Queried per launch these calls were most of the launch's host time.
+  struct Setup {
+    int busy[kMaxCluster + 1];
+    bool ready;
+  };
+  static Setup setups[kMaxDevicesScore];
+  static std::mutex mutex;
+  Setup own{};  // a device past the table is set up on every launch
+  Setup& su = dev >= 0 && dev < kMaxDevicesScore ? setups[dev] : own;
+  std::unique_lock<std::mutex> lock(mutex);
   cudaError_t err = cudaSuccess;
-  if (dev < kMaxDevicesScore && busy[dev][0] == 0) {
-    const size_t smem_q = C::smem_bytes(2 * NQ, kMaxCluster);
-    if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_q))) !=
-            cudaSuccess ||
+  if (!su.ready) {
+    int sms = 0, smem_max = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    for (int c = 1; c <= kMaxCluster; ++c) {
+      const int b = static_cast<int>(C::smem_bytes(2 * NQ, c));
+      smem_max = b > smem_max ? b : smem_max;
+    }
+    if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max)) != cudaSuccess ||
         (err = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
       return err;
     for (int c = 1; c <= kMaxCluster; ++c) {
       cudaLaunchConfig_t q = {};
       q.blockDim = dim3(kScThreads);
-      q.dynamicSmemBytes = smem_q;
+      q.dynamicSmemBytes = C::smem_bytes(2 * NQ, kMaxCluster);
       q.gridDim = dim3(static_cast<unsigned>(c * sms));
       cudaLaunchAttribute qa[1];
       qa[0].id = cudaLaunchAttributeClusterDimension;
@@ -900,20 +914,14 @@ cudaError_t launch_score_dq(const Shape& s, const CUtensorMap& kmap, const CUten
         cudaGetLastError();
         n = c <= 8 ? sms / c : 0;
       }
-      busy[dev][c] = n * c;
+      su.busy[c] = n * c;
     }
-    busy[dev][0] = 1;
+    su.ready = true;
   }
-  int fallback[kMaxCluster + 1] = {};
-  for (int c = 1; c <= 8; ++c) fallback[c] = (sms / c) * c;
-  const Plan plan = plan_score(a.L, 2 * NQ, dev < kMaxDevicesScore ? busy[dev] : fallback);
+  lock.unlock();
+  const Plan plan = plan_score(a.L, 2 * NQ, su.busy);
   const size_t smem = C::smem_bytes(2 * NQ, plan.csize);
   const int n_stages = C::stages(2 * NQ, plan.csize);
-  err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (err != cudaSuccess) return err;
-  if (plan.csize > 8 && (err = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) !=
-                            cudaSuccess)
-    return err;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kScThreads);
   cfg.dynamicSmemBytes = smem;
@@ -926,14 +934,10 @@ cudaError_t launch_score_dq(const Shape& s, const CUtensorMap& kmap, const CUten
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   // one resident wave of clusters, each looping over its share of the instances
-  cfg.gridDim = dim3(static_cast<unsigned>(plan.csize * sms));
-  if (cudaOccupancyMaxActiveClusters(&max_clusters, score_kernel<D, NQ, MEAN, CAUSAL, COMBINE>, &cfg) != cudaSuccess || max_clusters < 1) {
-    cudaGetLastError();
-    max_clusters = sms / plan.csize > 0 ? sms / plan.csize : 1;
-  }
+  const int max_clusters = su.busy[plan.csize] >= plan.csize ? su.busy[plan.csize] / plan.csize : 1;
   const int n_clusters = max_clusters < s.n_inst ? max_clusters : s.n_inst;
   cfg.gridDim = dim3(static_cast<unsigned>(n_clusters * plan.csize));
-  return cudaLaunchKernelEx(&cfg, score_kernel<D, NQ, MEAN, CAUSAL, COMBINE>, kmap, kmap32, qmap, s, a, plan, n_stages);
+  return cudaLaunchKernelEx(&cfg, kern, kmap, kmap32, qmap, s, a, plan, n_stages);
 }
 
 template <int D, bool MEAN, bool CAUSAL>
