@@ -162,12 +162,13 @@ cudaError_t launch_score_causal(const Shape& s, const CUtensorMap& kmap, const C
 cudaError_t launch_score_causal_mean(const Shape& s, const CUtensorMap& kmap, const CUtensorMap& kmap32,
                                      const CUtensorMap& qmap, const ScoreArgs& a, cudaStream_t st);
 
-cudaError_t launch_select_gather(const Shape& s, const float* r, int L, int budget, __nv_bfloat16* K,
-                                 __nv_bfloat16* V, int* kept, int* err, cudaStream_t st);
+// r: the instances' log2 scores; the call may overwrite each instance's first one.
+cudaError_t launch_select_gather(const Shape& s, float* r, int L, int budget, __nv_bfloat16* K, __nv_bfloat16* V,
+                                 int* kept, int* err, cudaStream_t st);
 // Per-instance lengths: the instances work[0 .. *n_work), instance e with Ls[e] rows (at most cap).
-cudaError_t launch_select_gather_ragged(const Shape& s, const float* r, const int* Ls, const int* work,
-                                        const int* n_work, int budget, __nv_bfloat16* K, __nv_bfloat16* V, int* kept,
-                                        int* err, cudaStream_t st);
+cudaError_t launch_select_gather_ragged(const Shape& s, float* r, const int* Ls, const int* work, const int* n_work,
+                                        int budget, __nv_bfloat16* K, __nv_bfloat16* V, int* kept, int* err,
+                                        cudaStream_t st);
 
 cudaError_t launch_keep_all(const Shape& s, int L, int budget, int* kept, cudaStream_t st);
 

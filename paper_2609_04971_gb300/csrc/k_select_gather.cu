@@ -1,5 +1,8 @@
 // Selection (Eq. 7 with the keep set of Algorithm 2) and in-place compaction
-// of K and V (Eq. 8), one CTA of 256 threads per instance.
+// of K and V (Eq. 8): one CTA of 256 threads per instance does both, or, when
+// that leaves the chip idle (see use_split), a selection kernel of 1024 threads
+// per instance is followed by a gather kernel with a CTA per 128-byte column
+// slice of each tensor.
 //
 // Selection: the log2 scores of the candidates [n_prefix, L - W) are mapped to
 // order-preserving uint32 keys in shared memory; a 4-pass MSB-first radix
@@ -25,56 +28,51 @@ namespace bkv {
 namespace {
 
 constexpr int kSgThreads = 256;
-constexpr int kSgWarps = kSgThreads / 32;
+constexpr int kSelThreads = 1024;  // selection of the split form
+constexpr int kHists = 8;          // histogram copies (one per warp, or shared by warps w, w + 8, ...)
 
-// Exclusive block-wide prefix count of `flag`; also returns the block total.
+// Exclusive block-wide prefix count of `flag` (T threads); also returns the block total.
+template <int T>
 __device__ __forceinline__ void block_count_scan(bool flag, int* wsum, int& excl, int& total) {
+  constexpr int kWarps = T / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned bal = __ballot_sync(0xffffffffu, flag);
   if (lane == 0) wsum[warp] = __popc(bal);
   __syncthreads();
   int before = 0, all = 0;
+  if constexpr (kWarps <= 8) {
 #pragma unroll
-  for (int w = 0; w < kSgWarps; ++w) {
-    const int c = wsum[w];
-    before += (w < warp) ? c : 0;
-    all += c;
+    for (int w = 0; w < kWarps; ++w) {
+      const int c = wsum[w];
+      before += (w < warp) ? c : 0;
+      all += c;
+    }
+  } else {  // lane w reads warp w's count
+    const int c = lane < kWarps ? wsum[lane] : 0;
+    before = __reduce_add_sync(0xffffffffu, lane < warp ? c : 0);
+    all = __reduce_add_sync(0xffffffffu, c);
   }
   excl = before + __popc(bal & ((1u << lane) - 1u));
   total = all;
   __syncthreads();
 }
 
-// work / n_work (per-instance lengths): block w compresses instance work[w], with Ls[work[w]] rows,
-// when w < *n_work; otherwise every block compresses its own instance from L rows.
-template <int D>
-__global__ void __launch_bounds__(kSgThreads) select_gather_kernel(Shape s, const float* __restrict__ r, int L,
-                                                                    int budget, __nv_bfloat16* K, __nv_bfloat16* V,
-                                                                    int* kept, const int* __restrict__ Ls,
-                                                                    const int* __restrict__ work,
-                                                                    const int* __restrict__ n_work, int* err) {
-  extern __shared__ __align__(16) uint32_t keys[];  // [L]
-  __shared__ uint32_t hist[kSgWarps][256];
+// Selection of one instance by NT threads (block-uniform arguments): kept rows, ascending, to kept_e in
+// global memory and over the consumed keys in shared memory ([L] words).  first: the first evicted row
+// (L when none).  False when a checked build finds the kept set's size wrong.
+template <int NT>
+__device__ __forceinline__ bool select_rows(const Shape& s, const float* r_e, int L, int budget, uint32_t* keys, int* kept_e,
+                                            int& first, int* err) {
+  __shared__ uint32_t hist[kHists][256];
   __shared__ uint32_t tot[256];
-  __shared__ int wsum[kSgWarps];
+  __shared__ int wsum[NT / 32];
   __shared__ uint32_t sh_prefix, sh_k;
   __shared__ int sh_first_evicted;
-
-  int e = blockIdx.x;
-  if (work) {
-    if (e >= *n_work) return;  // whole block
-    e = work[e];
-    if (!in_bounds(e, s.n_inst, err)) return;  // whole block: every thread read the same entries
-    L = Ls[e];
-    if (!in_bounds(L - 1, s.cap, err)) return;
-  }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c_lo = s.n_prefix, c_hi = L - s.W;
   const int k_sel = budget - s.n_prefix - s.W;
-  const float* r_e = r + static_cast<size_t>(e) * s.cap;
-  int* kept_e = kept + static_cast<size_t>(e) * budget;
 
-  for (int j = tid; j < L; j += kSgThreads) keys[j] = float_order_key(r_e[j]);
+  for (int j = tid; j < L; j += NT) keys[j] = float_order_key(r_e[j]);
   if (tid == 0) {
     sh_prefix = 0;
     sh_k = static_cast<uint32_t>(k_sel);
@@ -87,17 +85,17 @@ __global__ void __launch_bounds__(kSgThreads) select_gather_kernel(Shape s, cons
   if (k_sel > 0) {
     for (int pass = 0; pass < 4; ++pass) {
       const int shift = 24 - 8 * pass;
-      for (int i = tid; i < kSgWarps * 256; i += kSgThreads) (&hist[0][0])[i] = 0;
+      for (int i = tid; i < kHists * 256; i += NT) (&hist[0][0])[i] = 0;
       __syncthreads();
-      for (int j = c_lo + tid; j < c_hi; j += kSgThreads) {
+      for (int j = c_lo + tid; j < c_hi; j += NT) {
         const uint32_t key = keys[j];
-        if ((key & pmask) == prefix) atomicAdd(&hist[warp][(key >> shift) & 255u], 1u);
+        if ((key & pmask) == prefix) atomicAdd(&hist[warp % kHists][(key >> shift) & 255u], 1u);
       }
       __syncthreads();
       if (tid < 256) {
         uint32_t t = 0;
 #pragma unroll
-        for (int w = 0; w < kSgWarps; ++w) t += hist[w][tid];
+        for (int w = 0; w < kHists; ++w) t += hist[w][tid];
         tot[tid] = t;
       }
       __syncthreads();
@@ -141,17 +139,17 @@ __global__ void __launch_bounds__(kSgThreads) select_gather_kernel(Shape s, cons
   // kept indices go to global memory and, in place of the consumed keys, to shared memory
   int* kept_s = reinterpret_cast<int*>(keys);
   int run_tie = 0, run_keep = 0;
-  for (int base = 0; base < L; base += kSgThreads) {
+  for (int base = 0; base < L; base += NT) {
     const int j = base + tid;
     const bool in = j < L;
     const bool cand = in && j >= c_lo && j < c_hi;
     const uint32_t key = cand ? keys[j] : 0u;
     const bool tie = cand && key == T;
     int tie_excl, tie_total;
-    block_count_scan(tie, wsum, tie_excl, tie_total);  // also orders every read of keys[base..] before the writes
+    block_count_scan<NT>(tie, wsum, tie_excl, tie_total);  // also orders every read of keys[base..] before the writes
     const bool keep = in && (!cand || key > T || (tie && run_tie + tie_excl < k_ties));
     int keep_excl, keep_total;
-    block_count_scan(keep, wsum, keep_excl, keep_total);
+    block_count_scan<NT>(keep, wsum, keep_excl, keep_total);
     if (keep && in_bounds(run_keep + keep_excl, budget, err)) {
       kept_e[run_keep + keep_excl] = j;
       kept_s[run_keep + keep_excl] = j;  // position <= j: that key has been read already
@@ -162,8 +160,41 @@ __global__ void __launch_bounds__(kSgThreads) select_gather_kernel(Shape s, cons
     run_keep += keep_total;
   }
   __syncthreads();
+  first = sh_first_evicted;
   // the selection keeps exactly `budget` rows; a checked build verifies it (block-uniform)
-  if (!in_bounds(run_keep - budget, 1, err) || !in_bounds(budget - run_keep, 1, err)) return;
+  return in_bounds(run_keep - budget, 1, err) && in_bounds(budget - run_keep, 1, err);
+}
+
+
+// work / n_work (per-instance lengths): block w compresses instance work[w], with Ls[work[w]] rows,
+// when w < *n_work; otherwise every block compresses its own instance from L rows.  False: not this block.
+__device__ __forceinline__ bool block_instance(const Shape& s, int w, const int* Ls, const int* work, const int* n_work,
+                                               int& e, int& L, int* err) {
+  e = w;
+  if (work) {
+    if (e >= *n_work) return false;
+    e = work[e];
+    if (!in_bounds(e, s.n_inst, err)) return false;  // every thread read the same entries
+    L = Ls[e];
+    if (!in_bounds(L - 1, s.cap, err)) return false;
+  }
+  return true;
+}
+
+template <int D>
+__global__ void __launch_bounds__(kSgThreads) select_gather_kernel(Shape s, const float* __restrict__ r, int L,
+                                                                    int budget, __nv_bfloat16* K, __nv_bfloat16* V,
+                                                                    int* kept, const int* __restrict__ Ls,
+                                                                    const int* __restrict__ work,
+                                                                    const int* __restrict__ n_work, int* err) {
+  extern __shared__ __align__(16) uint32_t keys[];  // [L]
+  int e, first;
+  if (!block_instance(s, blockIdx.x, Ls, work, n_work, e, L, err)) return;  // whole block
+  const int tid = threadIdx.x;
+  if (!select_rows<kSgThreads>(s, r + static_cast<size_t>(e) * s.cap, L, budget, keys,
+                               kept + static_cast<size_t>(e) * budget, first, err))
+    return;
+  const int* kept_s = reinterpret_cast<const int*>(keys);
 
   // ---------------------------------------------------------------- in-place gather
   constexpr int kVpr = D * 2 / 16;                 // 16-byte vectors per row of one tensor
@@ -175,7 +206,6 @@ __global__ void __launch_bounds__(kSgThreads) select_gather_kernel(Shape s, cons
   const int row0 = tid / kRowVec;                  // first row of this thread inside a chunk
   uint4* base_t = reinterpret_cast<uint4*>((col < kVpr ? K : V) + static_cast<size_t>(e) * s.cap * D) +
                   (col < kVpr ? col : col - kVpr);
-  const int first = sh_first_evicted;
 
   uint4 cur[kPer], nxt[kPer];
   auto load_chunk = [&](int i0, uint4 (&R)[kPer]) {
@@ -207,6 +237,80 @@ __global__ void __launch_bounds__(kSgThreads) select_gather_kernel(Shape s, cons
   }
 }
 
+// ---- split form
+// Selection only.  The instance's first score, read by now, receives the first evicted row.
+__global__ void __launch_bounds__(kSelThreads) select_kernel(Shape s, float* r, int L, int budget, int* kept,
+                                                             const int* __restrict__ Ls, const int* __restrict__ work,
+                                                             const int* __restrict__ n_work, int* err) {
+  extern __shared__ __align__(16) uint32_t keys[];  // [L]
+  int e, first;
+  if (!block_instance(s, blockIdx.x, Ls, work, n_work, e, L, err)) return;  // whole block
+  float* r_e = r + static_cast<size_t>(e) * s.cap;
+  if (!select_rows<kSelThreads>(s, r_e, L, budget, keys, kept + static_cast<size_t>(e) * budget, first, err)) first = L;
+  if (threadIdx.x == 0) r_e[0] = __int_as_float(first);
+}
+
+// Gather of one 128-byte column slice of one tensor of one instance: columns are independent, so the
+// in-place rule (see the file comment) holds slice by slice.  A chunk is 256 rows, eight per thread; its
+// kept indices pass through shared memory two chunks ahead.
+template <int D>
+__global__ void __launch_bounds__(kSgThreads, 3) gather_kernel(Shape s, const float* __restrict__ r, int L, int budget,
+                                                            __nv_bfloat16* K, __nv_bfloat16* V,
+                                                            const int* __restrict__ kept, const int* __restrict__ Ls,
+                                                            const int* __restrict__ work,
+                                                            const int* __restrict__ n_work, int* err) {
+  constexpr int kSlices = 2 * D / 64;     // 128-byte slices of K, then of V
+  constexpr int kVpr = D * 2 / 16;        // 16-byte vectors per row of one tensor
+  constexpr int kPer = 8;
+  constexpr int kRows = kSgThreads / 8;   // rows per pass
+  constexpr int kChunkRows = kRows * kPer;
+  static_assert(kChunkRows == kSgThreads, "one kept index per thread and chunk");
+  __shared__ int idx[3][kChunkRows];
+  int e;
+  if (!block_instance(s, blockIdx.x / kSlices, Ls, work, n_work, e, L, err)) return;  // whole block
+  const int slice = blockIdx.x % kSlices, tid = threadIdx.x, row0 = tid >> 3;
+  const int first = __float_as_int(__ldcg(r + static_cast<size_t>(e) * s.cap));
+  const int* kept_e = kept + static_cast<size_t>(e) * budget;
+  const bool is_k = slice < kSlices / 2;
+  uint4* base = reinterpret_cast<uint4*>((is_k ? K : V) + static_cast<size_t>(e) * s.cap * D) +
+                (is_k ? slice : slice - kSlices / 2) * 8 + (tid & 7);
+  auto index = [&](int i0) { return i0 + tid < budget ? __ldcg(kept_e + i0 + tid) : 0; };
+  uint4 cur[kPer], nxt[kPer];
+  auto load_chunk = [&](int i0, const int* at, uint4 (&R)[kPer]) {
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const int row = i0 + row0 + kRows * u;
+      if (row < budget) {
+        int src = at[row0 + kRows * u];
+        if (!in_bounds(src - row, L - row, err)) src = row;  // kept rows satisfy row <= kept[row] < L
+        R[u] = __ldcg(base + static_cast<size_t>(src) * kVpr);
+      }
+    }
+  };
+  if (first >= budget) return;  // whole block: nothing moves
+  idx[0][tid] = index(first);
+  idx[1][tid] = index(first + kChunkRows);
+  int ahead = index(first + 2 * kChunkRows);
+  __syncthreads();
+  load_chunk(first, idx[0], cur);
+  int c = 0;  // chunk number modulo 3
+  for (int i0 = first; i0 < budget; i0 += kChunkRows) {
+    __syncthreads();  // every load of this chunk was issued before any of its stores; the next indices are there
+    const int c1 = c == 2 ? 0 : c + 1, c2 = c1 == 2 ? 0 : c1 + 1;
+    if (i0 + kChunkRows < budget) load_chunk(i0 + kChunkRows, idx[c1], nxt);
+    idx[c2][tid] = ahead;
+    ahead = index(i0 + 3 * kChunkRows);
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const int row = i0 + row0 + kRows * u;
+      if (row < budget) base[static_cast<size_t>(row) * kVpr] = cur[u];
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) cur[u] = nxt[u];
+    c = c1;
+  }
+}
+
 __global__ void keep_all_kernel(int n_inst, int L, int budget, int* kept) {
   const size_t n = static_cast<size_t>(n_inst) * budget;
   for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;
@@ -216,44 +320,52 @@ __global__ void keep_all_kernel(int n_inst, int L, int budget, int* kept) {
   }
 }
 
-template <int D>
-cudaError_t launch_sg_d(const Shape& s, const float* r, int L, int budget, __nv_bfloat16* K, __nv_bfloat16* V,
-                        int* kept, int* err, cudaStream_t st) {
-  const size_t smem = sizeof(uint32_t) * static_cast<size_t>(L);
-  const cudaError_t ce = cudaFuncSetAttribute(select_gather_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              static_cast<int>(smem));
-  if (ce != cudaSuccess) return ce;
-  select_gather_kernel<D><<<s.n_inst, kSgThreads, smem, st>>>(s, r, L, budget, K, V, kept, nullptr, nullptr, nullptr,
-                                                              err);
-  return cudaGetLastError();
+// Whether the split form is used for caches of up to L rows.  The fused kernel streams at the copy rate
+// while a few of its CTAs per SM overlap one's selection with the others' gathers; it does not when there
+// are too few, or when the keys of long caches (4 bytes a row) leave room for one per SM.  The split's
+// selection overlaps nothing, and it pays a launch, which caches of a few hundred rows do not win back.
+// Whole compress steps on 152 SMs, fused -> split: 288 instances of 4224 rows 294 -> 255 us, 512 of them
+// 392 -> 376; 1536 1750 -> 1766, 4608 4383 -> 4500; 288 instances of 32700 rows 3600 -> 3237 (the gather
+// 1700 -> 1345).
+bool use_split(int n_inst, int L, int budget, int sms) {
+  return budget >= 1024 && (n_inst <= 4 * sms || 2 * (sizeof(uint32_t) * static_cast<size_t>(L) + 12 * 1024) > 224 * 1024);
 }
 
-// L_max sizes the shared-memory key array (every instance has at most that many rows).
 template <int D>
-cudaError_t launch_sg_ragged_d(const Shape& s, const float* r, const int* Ls, const int* work, const int* n_work,
-                               int L_max, int budget, __nv_bfloat16* K, __nv_bfloat16* V, int* kept, int* err,
-                               cudaStream_t st) {
-  const size_t smem = sizeof(uint32_t) * static_cast<size_t>(L_max);
-  const cudaError_t ce = cudaFuncSetAttribute(select_gather_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              static_cast<int>(smem));
-  if (ce != cudaSuccess) return ce;
-  select_gather_kernel<D><<<s.n_inst, kSgThreads, smem, st>>>(s, r, L_max, budget, K, V, kept, Ls, work, n_work, err);
+cudaError_t launch_sg_d(const Shape& s, float* r, const int* Ls, const int* work, const int* n_work, int L, int budget,
+                        __nv_bfloat16* K, __nv_bfloat16* V, int* kept, int* err, cudaStream_t st) {
+  const size_t smem = sizeof(uint32_t) * static_cast<size_t>(L);  // every instance has at most L rows
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  if (use_split(s.n_inst, L, budget, sms)) {
+    e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+    select_kernel<<<s.n_inst, kSelThreads, smem, st>>>(s, r, L, budget, kept, Ls, work, n_work, err);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    gather_kernel<D><<<s.n_inst * (2 * D / 64), kSgThreads, 0, st>>>(s, r, L, budget, K, V, kept, Ls, work, n_work, err);
+    return cudaGetLastError();
+  }
+  e = cudaFuncSetAttribute(select_gather_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  select_gather_kernel<D><<<s.n_inst, kSgThreads, smem, st>>>(s, r, L, budget, K, V, kept, Ls, work, n_work, err);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_select_gather(const Shape& s, const float* r, int L, int budget, __nv_bfloat16* K,
-                                 __nv_bfloat16* V, int* kept, int* err, cudaStream_t st) {
-  return s.d == 128 ? launch_sg_d<128>(s, r, L, budget, K, V, kept, err, st)
-                    : launch_sg_d<64>(s, r, L, budget, K, V, kept, err, st);
+cudaError_t launch_select_gather(const Shape& s, float* r, int L, int budget, __nv_bfloat16* K, __nv_bfloat16* V,
+                                 int* kept, int* err, cudaStream_t st) {
+  return s.d == 128 ? launch_sg_d<128>(s, r, nullptr, nullptr, nullptr, L, budget, K, V, kept, err, st)
+                    : launch_sg_d<64>(s, r, nullptr, nullptr, nullptr, L, budget, K, V, kept, err, st);
 }
 
-cudaError_t launch_select_gather_ragged(const Shape& s, const float* r, const int* Ls, const int* work,
-                                        const int* n_work, int budget, __nv_bfloat16* K, __nv_bfloat16* V, int* kept,
-                                        int* err, cudaStream_t st) {
-  return s.d == 128 ? launch_sg_ragged_d<128>(s, r, Ls, work, n_work, s.cap, budget, K, V, kept, err, st)
-                    : launch_sg_ragged_d<64>(s, r, Ls, work, n_work, s.cap, budget, K, V, kept, err, st);
+cudaError_t launch_select_gather_ragged(const Shape& s, float* r, const int* Ls, const int* work, const int* n_work,
+                                        int budget, __nv_bfloat16* K, __nv_bfloat16* V, int* kept, int* err,
+                                        cudaStream_t st) {
+  return s.d == 128 ? launch_sg_d<128>(s, r, Ls, work, n_work, s.cap, budget, K, V, kept, err, st)
+                    : launch_sg_d<64>(s, r, Ls, work, n_work, s.cap, budget, K, V, kept, err, st);
 }
 
 cudaError_t launch_keep_all(const Shape& s, int L, int budget, int* kept, cudaStream_t st) {
