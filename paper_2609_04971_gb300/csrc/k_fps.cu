@@ -243,7 +243,7 @@ __device__ __forceinline__ float first_eps(int N, int chain, float u_norm) {
 // NW warps, MT 16-row tiles per warp (warp w takes tiles w, w + NW, ...).  Lane 4 g of a warp owns the
 // rows g and g + 8 of each of its tiles: their screening values stay in its registers.
 template <int D, int NW, int MT, bool RES>
-__global__ void __launch_bounds__(32 * NW, MT == 2 ? 24 / NW : 1)
+__global__ void __launch_bounds__(32 * NW, MT == 2 ? 24 / NW : MT == 4 ? 3 : 1)
     fps_init_kernel(const __nv_bfloat16* __restrict__ q, int N, int nb, float* __restrict__ cent,
                     double* __restrict__ sums, long long* __restrict__ counts) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -625,14 +625,15 @@ cudaError_t launch_fps_dr(const Shape& s, const __nv_bfloat16* q_init, int N, fl
   return cudaGetLastError();
 }
 
-// Up to 256 rows two tiles per warp, with four warps up to 128 rows so that short prompts (64 rows per
-// head under Continual FPS) run as many small CTAs; up to 4096 rows eight tiles per warp.  Rows that do
+// Four warps up to 256 rows, with two or four tiles each (eight warps of two tiles: 233 us instead of 227
+// on the shape above: what a pick costs a warp besides its tiles is paid twice); up to 4096 rows eight
+// tiles per warp.  Rows that do
 // not fit in shared memory are read from global memory (L2) in every pass.
 template <int D>
 cudaError_t launch_fps_d(const Shape& s, const __nv_bfloat16* q_init, int N, float* cent, double* sums,
                          long long* counts, cudaStream_t st) {
   if (N <= 128) return launch_fps_dr<D, 4, 2, true>(s, q_init, N, cent, sums, counts, st);
-  if (N <= 256) return launch_fps_dr<D, 8, 2, true>(s, q_init, N, cent, sums, counts, st);
+  if (N <= 256) return launch_fps_dr<D, 4, 4, true>(s, q_init, N, cent, sums, counts, st);
   if (N <= 2048 && fps_layout(N, D, 512, true).total <= kFpsResident)
     return launch_fps_dr<D, 16, 8, true>(s, q_init, N, cent, sums, counts, st);
   if (N <= 2048) return launch_fps_dr<D, 16, 8, false>(s, q_init, N, cent, sums, counts, st);
