@@ -27,7 +27,7 @@ struct bkv_ctx {
   float* cent = nullptr;
   double* sums = nullptr;
   long long* counts = nullptr;
-  unsigned long long* spill = nullptr;  // batched update: zero between calls (update_spill_words)
+  unsigned long long* upd_scratch = nullptr;  // batched update (update_scratch_words)
   bool state_ready = false;
   // Continual FPS (BKV_F_CONTINUAL_FPS): per-query-head buffers; cent / counts then hold each
   // compress's beacons ([n_inst][G * n_beacons] rows, count 1 or 0) for the scoring-query build
@@ -195,7 +195,7 @@ void free_all(bkv_ctx* c) {
   cudaFree(c->cent);
   cudaFree(c->sums);
   cudaFree(c->counts);
-  cudaFree(c->spill);
+  cudaFree(c->upd_scratch);
   cudaFree(c->cbuf);
   cudaFree(c->csize);
   cudaFree(c->qobs);
@@ -272,11 +272,11 @@ int bkv_create(const bkv_config* cfg, void* stream, bkv_ctx** out) {
   const size_t ni = static_cast<size_t>(s.n_inst);
   cudaError_t e = cudaSuccess;
   const size_t nh = static_cast<size_t>(c->n_heads);
-  const size_t n_spill = c->cfps ? 0 : bkv::update_spill_words(s);
+  const size_t n_scratch = c->cfps ? 0 : bkv::update_scratch_words(s);
   if ((e = dmalloc(&c->cent, ni * s.nb * s.d)) != cudaSuccess ||
       (e = dmalloc(&c->sums, c->cfps ? 0 : ni * s.nb * s.d)) != cudaSuccess ||
       (e = dmalloc(&c->counts, ni * s.nb)) != cudaSuccess ||
-      (e = dmalloc(&c->spill, n_spill)) != cudaSuccess ||
+      (e = dmalloc(&c->upd_scratch, n_scratch)) != cudaSuccess ||
       (e = dmalloc(&c->cbuf, nh * c->b_max * s.d)) != cudaSuccess ||
       (e = dmalloc(&c->csize, nh)) != cudaSuccess ||
       (e = dmalloc(&c->qobs, ni * s.n_obs_pad * s.d)) != cudaSuccess ||
@@ -294,7 +294,7 @@ int bkv_create(const bkv_config* cfg, void* stream, bkv_ctx** out) {
   }
   if ((e = cudaMemsetAsync(c->cent, 0, sizeof(float) * ni * s.nb * s.d + 0, c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->sums, 0, sizeof(double) * (c->cfps ? 1 : ni * s.nb * s.d), c->stream)) != cudaSuccess ||
-      (e = cudaMemsetAsync(c->spill, 0, sizeof(unsigned long long) * (n_spill ? n_spill : 1), c->stream)) != cudaSuccess ||
+      (e = cudaMemsetAsync(c->upd_scratch, 0, sizeof(unsigned long long) * (n_scratch ? n_scratch : 1), c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->csize, 0, sizeof(int) * (nh ? nh : 1), c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->counts, 0, sizeof(long long) * ni * s.nb, c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->err, 0, sizeof(int), c->stream)) != cudaSuccess) {
@@ -426,7 +426,7 @@ int bkv_update_beacons(bkv_ctx* ctx, const void* q_new, int32_t n_new, int32_t* 
   if (rc != BKV_OK) return rc;
   ProfScope ps(ctx, BKV_K_UPDATE);
   cudaError_t e = bkv::launch_update(s, qmap, static_cast<int>(box_rows), n_new,
-                                     ctx->cent, ctx->sums, ctx->counts, assign_out, ctx->spill, ctx->err, ctx->stream);
+                                     ctx->cent, ctx->sums, ctx->counts, assign_out, ctx->upd_scratch, ctx->err, ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "update launch");
   return BKV_OK;
 }

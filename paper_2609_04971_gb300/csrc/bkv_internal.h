@@ -59,11 +59,11 @@ cudaError_t launch_fps_init(const Shape& s, const __nv_bfloat16* q_init, int n_i
                             long long* counts, cudaStream_t st);
 
 // qmap: the new queries as [n_inst * G * n_new][d] bf16 in boxes of
-// [box_rows][64] (128-byte swizzle), box_rows = min(128, rows); spill: update_spill_words(s) zeros, which
-// the call leaves zero; err: device error word.
-size_t update_spill_words(const Shape& s);
+// [box_rows][64] (128-byte swizzle), box_rows = min(128, rows); scratch: update_scratch_words(s) words,
+// zero at first and left to the calls after that; err: device error word.
+size_t update_scratch_words(const Shape& s);
 cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows, int n_new, float* cent,
-                          double* sums, long long* counts, int* assign_out, unsigned long long* spill, int* err,
+                          double* sums, long long* counts, int* assign_out, unsigned long long* scratch, int* err,
                           cudaStream_t st);
 // A few queries per instance (G * n_new <= kUpdateSmallMaxRows, e.g. one decode step): one warp
 // per instance, the same decisions and sums as launch_update (k_update_small.cu).

@@ -11,14 +11,13 @@
 // bf16(c / |c| - c_hi), so dot_b = D1[:, b] + D1[:, nbp + b] carries the
 // unit-centroid dot to about 2^-16 |q| (bf16 x bf16 products are exact, the
 // accumulation is fp32).  When best and second-best dots differ by at most
-// 1e-4 |q| (about twice the bound on their difference's error: 2^-17 |q| per
-// dot from the hi/lo split, 128 fp32 accumulation steps; |q| is taken a few
+// 7e-5 |q| (kScreenMargin; the bound is 4.2e-5 |q|, and |q| is taken a few
 // percent too large), the query is re-decided exactly: the beacon maximising
 // (q . c_b) / |c_b| in double-float arithmetic (exact products, TwoSum
 // accumulation, 1 / |c_b| from a double-float sum of squares and one Newton
 // step, to about 2^-44 relative), which agrees with the cosine (q . c_b) /
 // (|q| |c_b|) evaluated in fp64 except at ties below ~1e-12 (the lowest beacon
-// wins ties).  Only beacons screened within 2e-4 |q| of the best enter that
+// wins ties).  Only beacons screened within 1.4e-4 |q| of the best enter that
 // comparison.  Zero queries and instances without a valid beacon give -1.
 //
 // Sums: Q^T x A, where A is the tile's one-hot assignment matrix (128 queries x
@@ -26,32 +25,35 @@
 // whole into one of two operands, the tile itself (|x| >= 2^(E-10), a multiple
 // of 2^(E-17)) or a second tile (smaller ones, multiples of 2^(E-27) for
 // |x| >= 2^(E-20)), whose sums over 128 rows stay below 2^24 grid steps, so the
-// fp32 accumulator never rounds.  The two sums of a (column, beacon) cell become
-// one 64-bit integer per tile, added up in a register per cell.  The few
-// elements outside [2^(E-20), 2^E) (one in ten tiles of normal data) are
-// zeroed in the operands and go to the fold as a list (past 32 per instance
-// through a global array of this CTA).  E comes from the largest |q| this CTA has seen (before that from
-// the centroids), never below -11, so that what the operands hold is exact
-// in fixed point with 40 fractional bits; the result does not depend on it.
-// The call's sum is then added once to the fp64 running sum, correctly rounded
-// (fold_sum, in integers: fp64 is slow on this part), and c = fp32(sum / count) to within one fp32 ulp from
-// double-float arithmetic on the sum's bits.
+// fp32 accumulator never rounds.  The two sums of a (column, beacon) cell are
+// integers, added up over the tiles in two registers.  The few elements outside
+// [2^(E-20), 2^E) (one in five tiles of normal data) are zeroed in the operands
+// and added as a list (past 32 per instance through a global array of this CTA).
+// E comes from the largest |q| this CTA has seen (before that from the
+// centroids), never below -11, so that what the operands hold is exact in fixed
+// point with 40 fractional bits; the result does not depend on it.
+//
+// The call's sums (int64, 40 fractional bits) and counts go to scratch, from where
+// update_fold_kernel adds them once to the fp64 running sums, correctly rounded
+// and without fp64 arithmetic (slow on this part), and forms c = fp32(sum / count)
+// to within one fp32 ulp from double-float arithmetic on the sum's bits.
 //
 // Warp roles (23 warps): warp 0 TMA producer; warp 1 TMEM allocation and the
 // screening MMAs; warp 2 the sums' MMAs; warps 3..10 two groups of four that
 // take alternate tiles, one query per thread (its decision, the split of its
 // elements, its column of A); warps 11..18 one column of d and half of the
-// beacons per thread: they take the sums out of tensor memory and fold them
-// into the running state; warps 19..22 build the unit-centroid operand of the
-// next instances.  All waits are bounded.
+// beacons per thread: they take the sums out of tensor memory; warps 19..22
+// build the unit-centroid operand of the next instances.  All waits are bounded.
 //
-// What bounds it: the roles' instruction streams.  About 9 K warp instructions per
-// tile at 40 % issue, a quarter of the stalls instruction fetch (hence the loops
-// kept small), with two tiles in flight per SM because shared memory holds no
-// third second-tile.  The sums took most of the time when they were formed in fp32
-// parts by CUDA cores from rows sorted by beacon (about 14 K warp instructions
-// per tile): 4608 instances x 512 queries of 128, 8 beacons: 393 us, now 298 (95 at
-// the copy rate); 8192 instances, 16 beacons: 815 us, now 537 (206).
+// What bounds it: a tile's chain through its group (dots, split, decision, sums:
+// about 8 K clocks, two tiles in flight per SM because shared memory holds no
+// third second-tile) and instruction fetch: the roles share the instruction caches,
+// so loops are kept rolled and rare paths small (re-decisions and spilled elements,
+// three tiles in ten, still cost a fifth of the time).  Sums formed in fp32 parts
+// by CUDA cores from rows sorted by beacon took about 14 K warp instructions per
+// tile.  With the fold kernel: 4608 instances x 512 queries of 128, 8 beacons: 393
+// us, now 255 (95 at the copy rate); 8192 instances, 16 beacons: 815 us, now 485
+// (206).
 #include "bkv_device.cuh"
 #include "bkv_internal.h"
 #include "k_update_math.cuh"
@@ -68,11 +70,15 @@ constexpr int kQTile = 128;                 // queries per tile (MMA M of the sc
 constexpr uint32_t kQBox = 128 * 128;       // [128 rows][64 bf16] swizzled box slot
 constexpr int kUMaxStages = 6;
 constexpr int kDots = 3;                    // screening accumulators in tensor memory
-constexpr int kSums = 4;                    // sum accumulators: a fold may take as long as its instance's tiles
+constexpr int kSums = 4;                    // sum accumulators in tensor memory
 constexpr int kSlots = 16;                  // per-instance words in flight between the roles (at most 11 instances)
 constexpr int kSpillSlots = 8;              // instances whose spilled elements may be in flight
 constexpr int kSpillList = 32;              // spilled elements per instance kept in shared memory
 constexpr size_t kUSmemBudget = 220 * 1024;
+// A query is re-decided exactly when its best and second-best dots differ by at most this fraction of |q|.
+// A screened dot is within 2^-18 |q| (the hi / lo split) + 136 * 2^-23 |q| (17 additions in each of eight
+// K = 16 steps) + 2^-21 |q| (1 / |c|) of the exact one, so a difference of two within 4.2e-5 |q|.
+constexpr float kScreenMargin = 7e-5f;
 constexpr int kMinE = -11, kMaxE = 14;
 constexpr int kLargeBits = 10;              // octaves below 2^E that the tile itself holds
 constexpr int kSmallBits = 20;              // octaves below 2^E that the operands hold
@@ -85,6 +91,8 @@ struct UpdArgs {
   long long* counts;
   int* assign_out;
   unsigned long long* spill;  // [grid][kSpillSlots][nb][D], zero between instances
+  long long* call_sum;        // [n_inst][nb][D]: this call's sums, units of 2^-40, for the fold kernel
+  int* call_cnt;              // [n_inst][nb]: queries assigned
   int* err;
 };
 
@@ -211,7 +219,7 @@ __device__ __noinline__ int refine_row(const unsigned char* raw, const unsigned 
       n2d = df_add(n2d, df_two_prod(c[j], c[j]));
       dt = df_add(dt, df_two_prod(x[j], c[j]));
     }
-#pragma unroll
+#pragma unroll 1  // few instructions: they are fetched cold
     for (int o = 16; o > 0; o >>= 1) {
       n2 += __shfl_xor_sync(0xffffffffu, n2, o);
       n2d = df_add(n2d, DF{__shfl_xor_sync(0xffffffffu, n2d.hi, o), __shfl_xor_sync(0xffffffffu, n2d.lo, o)});
@@ -266,7 +274,7 @@ __device__ __noinline__ bool spill_row(unsigned char* raw, unsigned char* small,
   const uint32_t hi = pow2_bf16x2(E) & 0xffffu, lo = pow2_bf16x2(E - kSmallBits) & 0xffffu;
   constexpr int kC = D / 32;  // this lane's columns
   bool over = false;
-#pragma unroll
+#pragma unroll 1  // few instructions: they are fetched cold
   for (int k = 0; k < kC; ++k) {
     const int col = lane * kC + k;
     const uint32_t off = sw128_offset(n, col, kQBox);
@@ -605,7 +613,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
 
       // ---- decision
       const bool wild = degenerate || !(qn2 > 1e-30f && qn2 < 1e30f);
-      const float margin = kMarginRel * sqrt_approx(qn2);
+      const float margin = kScreenMargin * sqrt_approx(qn2);
       const bool close = n < rows && vm != 0u && (wild || !(best - second > margin));
       int my_b = n < rows ? bi : -1;
       uint32_t need = __ballot_sync(0xffffffffu, close);
@@ -677,25 +685,15 @@ __global__ void __launch_bounds__(kUThreads, 1)
     for (int i = 0, g = 0; i < n_my; ++i) {
       const int e = blockIdx.x + i * gridDim.x, slot = i & (kSlots - 1);
       const size_t cells = static_cast<size_t>(nb) * D, cbase = static_cast<size_t>(e) * cells;
-      if (first_warp && lane == 0) bulk_prefetch_l2(a.sums + cbase, static_cast<uint32_t>(cells) * 8);
       // sums of the two operands, each below 2^24 per tile (d = 64: of one, by this thread's half); more than
       // kFlush tiles are passed on through the spill array
       constexpr int kFlush = 64;
       int acc_l[HB], acc_s[HB];
 #pragma unroll
       for (int b = 0; b < HB; ++b) acc_l[b] = acc_s[b] = 0;
-      const long long cnt_old = lane < nb ? a.counts[static_cast<size_t>(e) * nb + lane] : 0;
       bool ok = true;  // false after a wait gave up: the barriers below are still taken
-      constexpr int kChunk = 2;  // beacons folded at once (more would overlap more latency, but cost instruction cache)
-      double s_old[kChunk];      // running sums of the next chunk to fold
-      auto load_old = [&](int b0) {
-#pragma unroll
-        for (int u = 0; u < kChunk; ++u)
-          s_old[u] = b0 + u < nb && !small_half ? a.sums[cbase + static_cast<size_t>(b0 + u) * D + col] : 1.0;
-      };
       for (int t = 0; ok && t < T; ++t, ++g) {
         const int ub = g % kSums;
-        if (t == T - 1) load_old(h0);  // ahead of the last tile's sums
         ok = mbar_wait(&cntready[ub], (g / kSums) & 1, abort_flag, a.err, kDevTimeoutEpilogue) &&
              mbar_wait(&sumfull[ub], (g / kSums) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
         ok = __all_sync(0xffffffffu, ok);
@@ -742,10 +740,8 @@ __global__ void __launch_bounds__(kUThreads, 1)
       }
       if (T > kFlush) named_barrier(1, 256);  // what another warp passed on (d = 64) is there
 
-      // ---- fold this instance's sums into the running state
+      // ---- this instance's sums of the call, for the fold kernel
       const int add = lane < nb ? add_cnt[slot][lane] : 0;
-      const uint32_t touched = ok ? __ballot_sync(0xffffffffu, add > 0) : 0u;
-      const DF rcp = count_reciprocal(add > 0 ? cnt_old + add : 1);  // lane b: beacon b
       const int shift = static_cast<signed char>(exp_sh[slot] & 0xff) + 40 - (kSmallBits + 7);  // to units of 2^-40
       const bool spilled = spilled_sh[slot] != 0;
       const SpillList& list = list_sh[i & (kSpillSlots - 1)];
@@ -761,77 +757,24 @@ __global__ void __launch_bounds__(kUThreads, 1)
 #pragma unroll
           for (int b = 0; b < HB; ++b) acc_s[b] = xchg[(h0 + b) * 64 + col];
       }
-#pragma unroll 1
-      for (int b0 = h0; b0 < nb && b0 < h0 + HB; b0 += kChunk) {  // chunk b0 sits in acc_*[0 .. kChunk)
-        double s_in[kChunk];
-        long long f[kChunk];
-        bool mine[kChunk];
+      long long* out = a.call_sum + cbase + static_cast<size_t>(h0) * D + col;
+      if (ok && !small_half) {
 #pragma unroll
-        for (int u = 0; u < kChunk; ++u) {
-          const int b = b0 + u;
-          mine[u] = b < nb && ((touched >> (b & 31)) & 1u) && !small_half;
-          s_in[u] = mine[u] ? s_old[u] : 1.0;
-          f[u] = mine[u] ? (acc_l[u] * 1024ll + acc_s[u]) << shift : 0;
-          if (mine[u] && spilled) {
-            f[u] += static_cast<long long>(__ldcg(spill + b * D + col));
-            spill[b * D + col] = 0ull;
+        for (int b = 0; b < HB; ++b)
+          if (h0 + b < nb) out[b * D] = (acc_l[b] * 1024ll + acc_s[b]) << shift;
+        for (int k = 0; k < n_list; ++k) {  // spilled elements of this thread's cells: rare
+          const int b = (list.key[k] >> 8) - h0;
+          if ((list.key[k] & 0xff) == col && b >= 0 && b < HB) out[b * D] += list.val[k];
+        }
+        if (spilled)
+          for (int b = 0; b < HB && h0 + b < nb; ++b) {
+            out[b * D] += static_cast<long long>(__ldcg(spill + (h0 + b) * D + col));
+            spill[(h0 + b) * D + col] = 0ull;
           }
-        }
-        if (b0 + kChunk < h0 + HB) load_old(b0 + kChunk);
-        for (int k = 0; k < n_list; ++k) {
-          const int rel = list.key[k] - ((b0 << 8) | col);  // (beacon - b0) << 8 where the column is this thread's
-#pragma unroll
-          for (int u = 0; u < kChunk; ++u)
-            if (rel == u << 8 && mine[u]) f[u] += list.val[k];
-        }
-        // the common case for the chunk at once (the cells' latencies overlap), the rest one by one
-        double s_new[kChunk];
-        float c_new[kChunk];
-        bool plain = true;
-#pragma unroll
-        for (int u = 0; u < kChunk; ++u) {
-          const int b = (b0 + u) & 31;
-          const DF rb{__shfl_sync(0xffffffffu, rcp.hi, b), __shfl_sync(0xffffffffu, rcp.lo, b)};
-          plain &= fold_and_centroid(s_in[u], f[u], rb, s_new[u], c_new[u]);
-        }
-        if (!plain) {
-#pragma unroll 1
-          for (int u = 0; u < kChunk; ++u) {
-            const int b = (b0 + u) & 31;
-            DF rb = count_reciprocal(1);
-            if (b < nb && add_cnt[slot][b] > 0) rb = count_reciprocal(a.counts[static_cast<size_t>(e) * nb + b] + add_cnt[slot][b]);
-            double so = s_in[0];
-            long long fu = f[0];
-#pragma unroll
-            for (int k = 1; k < kChunk; ++k) {
-              so = k == u ? s_in[k] : so;
-              fu = k == u ? f[k] : fu;
-            }
-            const double sn = fold_sum(so, fu);
-            const float cn = centroid_value(sn, rb);
-#pragma unroll
-            for (int k = 0; k < kChunk; ++k) {
-              s_new[k] = k == u ? sn : s_new[k];
-              c_new[k] = k == u ? cn : c_new[k];
-            }
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < kChunk; ++u)
-          if (mine[u]) {
-            const size_t gi = cbase + static_cast<size_t>(b0 + u) * D + col;
-            a.sums[gi] = s_new[u];
-            a.cent[gi] = c_new[u];
-          }
-#pragma unroll
-        for (int b = 0; b + kChunk < HB; ++b) {
-          acc_l[b] = acc_l[b + kChunk];
-          acc_s[b] = acc_s[b + kChunk];
-        }
       }
       if (spilled) __threadfence();
-      named_barrier(1, 256);  // every warp has read this slot's words, the counts (and, d = 64, the exchanged sums)
-      if (ok && first_warp && add > 0) a.counts[static_cast<size_t>(e) * nb + lane] = cnt_old + add;
+      named_barrier(1, 256);  // every warp has read this slot's words (and, d = 64, the exchanged sums)
+      if (ok && first_warp && lane < nb) a.call_cnt[static_cast<size_t>(e) * nb + lane] = add;
       if (first_warp) add_cnt[slot][lane] = 0;
       if (first_warp && lane == 0) {
         spilled_sh[slot] = 0;
@@ -924,6 +867,61 @@ __global__ void __launch_bounds__(kUThreads, 1)
   }
 }
 
+// The call's sums into the running state: thread = (instance, column), its beacons in fours.  A kernel of
+// its own: as a role of update_kernel its instructions kept the other roles waiting for theirs (4608
+// instances of 8 beacons 298 -> 270 us, 8192 of 16 537 -> 516 us, this kernel included).  What bounds it:
+// 28 bytes and about 130 instructions per cell.
+constexpr int kFoldThreads = 128;
+template <int D>
+__global__ void __launch_bounds__(kFoldThreads) update_fold_kernel(int n_inst, int nb, const long long* __restrict__ call_sum,
+                                                                   const int* __restrict__ call_cnt, float* cent,
+                                                                   double* sums, long long* counts) {
+  constexpr int kPer = kFoldThreads / D;  // instances per block
+  constexpr int kChunk = 4;
+  __shared__ DF rcp[kPer][kMaxBeacons];
+  __shared__ int added[kPer][kMaxBeacons];
+  const int sub = threadIdx.x / D, col = threadIdx.x % D;
+  const int e = blockIdx.x * kPer + sub;
+  if (e < n_inst && col < nb) {
+    const size_t i = static_cast<size_t>(e) * nb + col;
+    const int add = call_cnt[i];
+    added[sub][col] = add;
+    if (add > 0) {
+      const long long n = counts[i] + add;
+      counts[i] = n;
+      rcp[sub][col] = count_reciprocal(n);
+    }
+  }
+  __syncthreads();
+  if (e >= n_inst) return;
+  const size_t base = static_cast<size_t>(e) * nb * D + col;
+  for (int b0 = 0; b0 < nb; b0 += kChunk) {
+    double s_old[kChunk], s_new[kChunk];
+    long long f[kChunk];
+    float c_new[kChunk];
+    bool mine[kChunk], ok[kChunk];
+#pragma unroll
+    for (int u = 0; u < kChunk; ++u) {
+      mine[u] = b0 + u < nb && added[sub][b0 + u < nb ? b0 + u : 0] > 0;
+      s_old[u] = mine[u] ? sums[base + static_cast<size_t>(b0 + u) * D] : 1.0;
+      f[u] = mine[u] ? __ldcs(call_sum + base + static_cast<size_t>(b0 + u) * D) : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < kChunk; ++u)
+      ok[u] = fold_and_centroid(s_old[u], f[u], rcp[sub][b0 + u < nb ? b0 + u : 0], s_new[u], c_new[u]);
+#pragma unroll
+    for (int u = 0; u < kChunk; ++u)
+      if (mine[u]) {
+        if (!ok[u]) {  // a sum off the 2^-40 grid, past 2^22 or zero
+          s_new[u] = fold_sum(s_old[u], f[u]);
+          c_new[u] = centroid_value(s_new[u], rcp[sub][b0 + u]);
+        }
+        sums[base + static_cast<size_t>(b0 + u) * D] = s_new[u];
+        cent[base + static_cast<size_t>(b0 + u) * D] = c_new[u];
+      }
+  }
+}
+
 template <int D, int NBO>
 cudaError_t launch_update_dn(const UpdArgs& a, const CUtensorMap& qmap, int grid, cudaStream_t st) {
   using C = UpdCfg<D, NBO>;
@@ -932,6 +930,11 @@ cudaError_t launch_update_dn(const UpdArgs& a, const CUtensorMap& qmap, int grid
       cudaFuncSetAttribute(update_kernel<D, NBO>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   update_kernel<D, NBO><<<grid, kUThreads, smem, st>>>(qmap, a, C::stages(a.nbp));
+  const cudaError_t le = cudaGetLastError();
+  if (le != cudaSuccess) return le;
+  constexpr int kPer = kFoldThreads / D;
+  update_fold_kernel<D><<<(a.n_inst + kPer - 1) / kPer, kFoldThreads, 0, st>>>(a.n_inst, a.nb, a.call_sum, a.call_cnt,
+                                                                              a.cent, a.sums, a.counts);
   return cudaGetLastError();
 }
 
@@ -944,12 +947,15 @@ int update_grid(int n_inst) {
 
 }  // namespace
 
-size_t update_spill_words(const Shape& s) {
-  return s.nb == 0 ? 0 : static_cast<size_t>(update_grid(s.n_inst)) * kSpillSlots * s.nb * s.d;
+// spill, then the call's sums, then its counts
+size_t update_scratch_words(const Shape& s) {
+  if (s.nb == 0) return 0;
+  const size_t inst = static_cast<size_t>(s.n_inst) * s.nb;
+  return static_cast<size_t>(update_grid(s.n_inst)) * kSpillSlots * s.nb * s.d + inst * s.d + (inst + 1) / 2;
 }
 
 cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows, int n_new,
-                          float* cent, double* sums, long long* counts, int* assign_out, unsigned long long* spill,
+                          float* cent, double* sums, long long* counts, int* assign_out, unsigned long long* scratch,
                           int* err, cudaStream_t st) {
   UpdArgs a;
   a.n_inst = s.n_inst;
@@ -961,9 +967,12 @@ cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows,
   a.sums = sums;
   a.counts = counts;
   a.assign_out = assign_out;
-  a.spill = spill;
-  a.err = err;
   const int grid = update_grid(s.n_inst);
+  const size_t inst = static_cast<size_t>(s.n_inst) * s.nb;
+  a.spill = scratch;
+  a.call_sum = reinterpret_cast<long long*>(scratch + static_cast<size_t>(grid) * kSpillSlots * s.nb * s.d);
+  a.call_cnt = reinterpret_cast<int*>(a.call_sum + inst * s.d);
+  a.err = err;
   if (s.d == 128)
     return s.nb <= 16 ? launch_update_dn<128, 16>(a, qmap, grid, st) : launch_update_dn<128, 32>(a, qmap, grid, st);
   return s.nb <= 16 ? launch_update_dn<64, 16>(a, qmap, grid, st) : launch_update_dn<64, 32>(a, qmap, grid, st);
