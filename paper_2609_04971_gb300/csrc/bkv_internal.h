@@ -30,6 +30,25 @@ constexpr int kMaxWindow = 64;
 constexpr int kMaxCapacity = 32768;
 constexpr int kMaxFpsRows = 4096;
 
+// Launch of a kernel that may be scheduled while the kernel before it on the stream finishes (programmatic
+// dependent launch): its launch latency and prologue overlap that kernel's tail.  The kernel calls
+// grid_dependency_wait before it touches global memory.
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                                    A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // ---- Continual FPS buffers (k_cfps.cu)
 constexpr int kCfpsMaxRows = 32;  // b_max = n_beacons + window per query head
 enum { kCfpsUpdate = 0, kCfpsBeacons = 1, kCfpsMerge = 2 };

@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(kQobsThreads) qobs_kernel(Shape s, const __nv_
                                                              __nv_bfloat16* __restrict__ qobs,
                                                              uint32_t* __restrict__ valid, int* err) {
   int e = blockIdx.x;
+  grid_dependency_wait();
   if (work) {
     if (e >= *n_work) return;  // whole block
     e = work[e];
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(64) rope_table_kernel(const __grid_constant__ 
                                                         int h, int rotate, double2* table, size_t row_stride, int* gaps,
                                                         int gap_max) {
   const int row = blockIdx.x / (W + 1), slot = blockIdx.x % (W + 1), i = threadIdx.x;
+  grid_dependency_wait();  // an earlier compress may still read the table
   const long long pos = c.pos[blockIdx.x];
   if (rotate) {
     double2* tab = table + static_cast<size_t>(first_row + row) * row_stride;
@@ -170,8 +172,8 @@ cudaError_t launch_rope_chunks(int W, int h, int rows, const double* inv_freq, c
       for (int w = 0; w < W; ++w) pos[w] = recent_pos[static_cast<size_t>(r0 + r) * W + w];
       pos[W] = t_pos[r0 + r];
     }
-    rope_table_kernel<N><<<n * (W + 1), h, 0, st>>>(c, r0, W, h, rotate, table, row_stride, gaps, gap_max);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_dependent(rope_table_kernel<N>, static_cast<unsigned>(n * (W + 1)), static_cast<unsigned>(h),
+                                           0, st, c, r0, W, h, rotate, table, row_stride, gaps, gap_max);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -197,18 +199,16 @@ cudaError_t launch_rope_table(int W, int h, int rows, const double* inv_freq, co
 cudaError_t launch_qobs(const Shape& s, const __nv_bfloat16* q_recent, const float* cent, const long long* counts,
                         const double2* rope, int rotate, __nv_bfloat16* qobs, uint32_t* valid, int* err,
                         cudaStream_t st) {
-  qobs_kernel<<<s.n_inst, kQobsThreads, 0, st>>>(s, q_recent, cent, counts, rope, 0, rotate, nullptr, nullptr, qobs,
-                                                 valid, err);
-  return cudaGetLastError();
+  return launch_dependent(qobs_kernel, static_cast<unsigned>(s.n_inst), kQobsThreads, 0, st, s, q_recent, cent, counts,
+                          rope, static_cast<size_t>(0), rotate, nullptr, nullptr, qobs, valid, err);
 }
 
 cudaError_t launch_qobs_ragged(const Shape& s, const __nv_bfloat16* q_recent, const float* cent,
                                const long long* counts, const double2* rope, size_t rope_row, int rotate,
                                const int* work, const int* n_work, __nv_bfloat16* qobs, uint32_t* valid, int* err,
                                cudaStream_t st) {
-  qobs_kernel<<<s.n_inst, kQobsThreads, 0, st>>>(s, q_recent, cent, counts, rope, rope_row, rotate, work, n_work,
-                                                 qobs, valid, err);
-  return cudaGetLastError();
+  return launch_dependent(qobs_kernel, static_cast<unsigned>(s.n_inst), kQobsThreads, 0, st, s, q_recent, cent, counts,
+                          rope, rope_row, rotate, work, n_work, qobs, valid, err);
 }
 
 }  // namespace bkv

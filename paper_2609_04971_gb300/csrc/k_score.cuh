@@ -404,6 +404,7 @@ __global__ void __launch_bounds__(kScThreads, 1)
   const int crank = csize > 1 ? static_cast<int>(cluster_ctarank()) : 0;
   const int cluster_id = blockIdx.x / csize;
   const int n_clusters = gridDim.x / csize;
+  grid_dependency_wait();
   int n_items = a.work ? *a.n_work : s.n_inst;  // instances to compress
   if (!in_bounds(n_items, s.n_inst + 1, a.err)) n_items = 0;
   const int n_my = cluster_id < n_items ? (n_items - cluster_id + n_clusters - 1) / n_clusters : 0;
@@ -926,13 +927,15 @@ cudaError_t launch_score_dq(const Shape& s, const CUtensorMap& kmap, const CUten
   cfg.blockDim = dim3(kScThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = static_cast<unsigned>(plan.csize);
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_dependent
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   // one resident wave of clusters, each looping over its share of the instances
   const int max_clusters = su.busy[plan.csize] >= plan.csize ? su.busy[plan.csize] / plan.csize : 1;
   const int n_clusters = max_clusters < s.n_inst ? max_clusters : s.n_inst;

@@ -170,6 +170,7 @@ __device__ __forceinline__ bool select_rows(const Shape& s, const float* r_e, in
 // when w < *n_work; otherwise every block compresses its own instance from L rows.  False: not this block.
 __device__ __forceinline__ bool block_instance(const Shape& s, int w, const int* Ls, const int* work, const int* n_work,
                                                int& e, int& L, int* err) {
+  grid_dependency_wait();
   e = w;
   if (work) {
     if (e >= *n_work) return false;
@@ -342,15 +343,16 @@ cudaError_t launch_sg_d(const Shape& s, float* r, const int* Ls, const int* work
   if (use_split(s.n_inst, L, budget, sms)) {
     e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    select_kernel<<<s.n_inst, kSelThreads, smem, st>>>(s, r, L, budget, kept, Ls, work, n_work, err);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    gather_kernel<D><<<s.n_inst * (2 * D / 64), kSgThreads, 0, st>>>(s, r, L, budget, K, V, kept, Ls, work, n_work, err);
-    return cudaGetLastError();
+    e = launch_dependent(select_kernel, static_cast<unsigned>(s.n_inst), kSelThreads, smem, st, s, r, L, budget, kept, Ls,
+                         work, n_work, err);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(gather_kernel<D>, static_cast<unsigned>(s.n_inst * (2 * D / 64)), kSgThreads, 0, st, s, r, L,
+                            budget, K, V, kept, Ls, work, n_work, err);
   }
   e = cudaFuncSetAttribute(select_gather_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  select_gather_kernel<D><<<s.n_inst, kSgThreads, smem, st>>>(s, r, L, budget, K, V, kept, Ls, work, n_work, err);
-  return cudaGetLastError();
+  return launch_dependent(select_gather_kernel<D>, static_cast<unsigned>(s.n_inst), kSgThreads, smem, st, s, r, L, budget,
+                          K, V, kept, Ls, work, n_work, err);
 }
 
 }  // namespace

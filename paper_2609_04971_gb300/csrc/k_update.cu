@@ -882,6 +882,7 @@ __global__ void __launch_bounds__(kFoldThreads) update_fold_kernel(int n_inst, i
   __shared__ int added[kPer][kMaxBeacons];
   const int sub = threadIdx.x / D, col = threadIdx.x % D;
   const int e = blockIdx.x * kPer + sub;
+  grid_dependency_wait();
   if (e < n_inst && col < nb) {
     const size_t i = static_cast<size_t>(e) * nb + col;
     const int add = call_cnt[i];
@@ -933,9 +934,8 @@ cudaError_t launch_update_dn(const UpdArgs& a, const CUtensorMap& qmap, int grid
   const cudaError_t le = cudaGetLastError();
   if (le != cudaSuccess) return le;
   constexpr int kPer = kFoldThreads / D;
-  update_fold_kernel<D><<<(a.n_inst + kPer - 1) / kPer, kFoldThreads, 0, st>>>(a.n_inst, a.nb, a.call_sum, a.call_cnt,
-                                                                              a.cent, a.sums, a.counts);
-  return cudaGetLastError();
+  return launch_dependent(update_fold_kernel<D>, static_cast<unsigned>((a.n_inst + kPer - 1) / kPer), kFoldThreads, 0, st,
+                          a.n_inst, a.nb, a.call_sum, a.call_cnt, a.cent, a.sums, a.counts);
 }
 
 int update_grid(int n_inst) {
