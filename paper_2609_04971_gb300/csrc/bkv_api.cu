@@ -27,7 +27,7 @@ struct bkv_ctx {
   float* cent = nullptr;
   double* sums = nullptr;
   long long* counts = nullptr;
-  unsigned long long* upd_scratch = nullptr;  // batched update (update_scratch_words)
+  unsigned long long* spill = nullptr;  // batched update: zero between calls (update_spill_words)
   bool state_ready = false;
   // Continual FPS (BKV_F_CONTINUAL_FPS): per-query-head buffers; cent / counts then hold each
   // compress's beacons ([n_inst][G * n_beacons] rows, count 1 or 0) for the scoring-query build
@@ -38,7 +38,7 @@ struct bkv_ctx {
   // scratch
   __nv_bfloat16* qobs = nullptr;  // [n_inst][n_obs_pad][d]
   uint32_t* valid = nullptr;      // [n_inst][4]
-  float* rscore = nullptr;        // [n_inst][cap]
+  float* rscore = nullptr;        // [n_inst][cap] (and the batched update's sums)
   double2* rope = nullptr;        // [W + 1][d / 2] fp64 (cos, sin), then the same table in fp32
   int* err = nullptr;             // device error word
   double inv_freq[64] = {};       // theta^(-2i / d), i < d / 2
@@ -195,7 +195,7 @@ void free_all(bkv_ctx* c) {
   cudaFree(c->cent);
   cudaFree(c->sums);
   cudaFree(c->counts);
-  cudaFree(c->upd_scratch);
+  cudaFree(c->spill);
   cudaFree(c->cbuf);
   cudaFree(c->csize);
   cudaFree(c->qobs);
@@ -272,16 +272,18 @@ int bkv_create(const bkv_config* cfg, void* stream, bkv_ctx** out) {
   const size_t ni = static_cast<size_t>(s.n_inst);
   cudaError_t e = cudaSuccess;
   const size_t nh = static_cast<size_t>(c->n_heads);
-  const size_t n_scratch = c->cfps ? 0 : bkv::update_scratch_words(s);
+  // the compress's scores; a batched update's sums use the same memory (neither outlives its call)
+  const size_t n_rscore = std::max(ni * s.cap, c->cfps ? 0 : (bkv::update_call_bytes(s) + 3) / 4);
+  const size_t n_spill = c->cfps ? 0 : bkv::update_spill_words(s);
   if ((e = dmalloc(&c->cent, ni * s.nb * s.d)) != cudaSuccess ||
       (e = dmalloc(&c->sums, c->cfps ? 0 : ni * s.nb * s.d)) != cudaSuccess ||
       (e = dmalloc(&c->counts, ni * s.nb)) != cudaSuccess ||
-      (e = dmalloc(&c->upd_scratch, n_scratch)) != cudaSuccess ||
+      (e = dmalloc(&c->spill, n_spill)) != cudaSuccess ||
       (e = dmalloc(&c->cbuf, nh * c->b_max * s.d)) != cudaSuccess ||
       (e = dmalloc(&c->csize, nh)) != cudaSuccess ||
       (e = dmalloc(&c->qobs, ni * s.n_obs_pad * s.d)) != cudaSuccess ||
       (e = dmalloc(&c->valid, ni * 4)) != cudaSuccess ||
-      (e = dmalloc(&c->rscore, ni * s.cap)) != cudaSuccess ||
+      (e = dmalloc(&c->rscore, n_rscore)) != cudaSuccess ||
       (e = dmalloc(&c->rope, static_cast<size_t>(s.W + 1) * (s.d / 2) * 3 / 2 + 1)) != cudaSuccess ||
       (e = dmalloc(&c->work, ni)) != cudaSuccess || (e = dmalloc(&c->n_work, 1)) != cudaSuccess ||
       (e = dmalloc(&c->rag, c->rag_bytes)) != cudaSuccess ||
@@ -294,7 +296,7 @@ int bkv_create(const bkv_config* cfg, void* stream, bkv_ctx** out) {
   }
   if ((e = cudaMemsetAsync(c->cent, 0, sizeof(float) * ni * s.nb * s.d + 0, c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->sums, 0, sizeof(double) * (c->cfps ? 1 : ni * s.nb * s.d), c->stream)) != cudaSuccess ||
-      (e = cudaMemsetAsync(c->upd_scratch, 0, sizeof(unsigned long long) * (n_scratch ? n_scratch : 1), c->stream)) != cudaSuccess ||
+      (e = cudaMemsetAsync(c->spill, 0, sizeof(unsigned long long) * (n_spill ? n_spill : 1), c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->csize, 0, sizeof(int) * (nh ? nh : 1), c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->counts, 0, sizeof(long long) * ni * s.nb, c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->err, 0, sizeof(int), c->stream)) != cudaSuccess) {
@@ -426,7 +428,7 @@ int bkv_update_beacons(bkv_ctx* ctx, const void* q_new, int32_t n_new, int32_t* 
   if (rc != BKV_OK) return rc;
   ProfScope ps(ctx, BKV_K_UPDATE);
   cudaError_t e = bkv::launch_update(s, qmap, static_cast<int>(box_rows), n_new,
-                                     ctx->cent, ctx->sums, ctx->counts, assign_out, ctx->upd_scratch, ctx->err, ctx->stream);
+                                     ctx->cent, ctx->sums, ctx->counts, assign_out, ctx->spill, ctx->rscore, ctx->err, ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "update launch");
   return BKV_OK;
 }
@@ -801,6 +803,8 @@ int bkv_sync(bkv_ctx* ctx) {
     return cuda_fail(ctx, e, "error word read");
   if (h != 0) {
     cudaMemset(ctx->err, 0, sizeof(int));
+    // an update that gave up a wait may have left its spill words set
+    if (!ctx->cfps) cudaMemset(ctx->spill, 0, sizeof(unsigned long long) * bkv::update_spill_words(ctx->shape));
     if (h == bkv::kDevBadLength)
       return fail(ctx, BKV_EINVAL, "a per-instance cache length was outside 1..capacity; that instance was left untouched");
     if (h == bkv::kDevBounds)

@@ -7,6 +7,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+#include <mutex>
+
 namespace bkv {
 
 // Per-context shape, derived once from bkv_config.
@@ -29,6 +32,37 @@ constexpr int kMaxObs = 128;
 constexpr int kMaxWindow = 64;
 constexpr int kMaxCapacity = 32768;
 constexpr int kMaxFpsRows = 4096;
+
+// Streaming multiprocessors of the current device (asked once per device; 0 on an error).
+inline int device_sms() {
+  static std::atomic<int> known[64];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  const bool in_table = dev >= 0 && dev < 64;
+  if (in_table && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  if (in_table) known[dev].store(n, std::memory_order_relaxed);
+  return n;
+}
+
+// Lets kernel kKern take `bytes` of dynamic shared memory on the current device.  The limit is only ever
+// raised, and only asked for above what every kernel may take (48 KB with its static part): small
+// launches are bound by such calls.
+template <auto kKern>
+cudaError_t allow_smem(size_t bytes) {
+  if (bytes <= 36 * 1024) return cudaSuccess;
+  static std::mutex mutex;
+  static size_t allowed[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mutex);
+  const bool in_table = dev >= 0 && dev < 64;
+  if (in_table && allowed[dev] >= bytes) return cudaSuccess;
+  e = cudaFuncSetAttribute(kKern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  if (e == cudaSuccess && in_table) allowed[dev] = bytes;
+  return e;
+}
 
 // Launch of a kernel that may be scheduled while the kernel before it on the stream finishes (programmatic
 // dependent launch): its launch latency and prologue overlap that kernel's tail.  The kernel calls
@@ -78,11 +112,12 @@ cudaError_t launch_fps_init(const Shape& s, const __nv_bfloat16* q_init, int n_i
                             long long* counts, cudaStream_t st);
 
 // qmap: the new queries as [n_inst * G * n_new][d] bf16 in boxes of
-// [box_rows][64] (128-byte swizzle), box_rows = min(128, rows); scratch: update_scratch_words(s) words,
-// zero at first and left to the calls after that; err: device error word.
-size_t update_scratch_words(const Shape& s);
+// [box_rows][64] (128-byte swizzle), box_rows = min(128, rows); spill: update_spill_words(s) zeros, which
+// the call leaves zero; call: update_call_bytes(s) of scratch; err: device error word.
+size_t update_spill_words(const Shape& s);
+size_t update_call_bytes(const Shape& s);
 cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows, int n_new, float* cent,
-                          double* sums, long long* counts, int* assign_out, unsigned long long* scratch, int* err,
+                          double* sums, long long* counts, int* assign_out, unsigned long long* spill, void* call, int* err,
                           cudaStream_t st);
 // A few queries per instance (G * n_new <= kUpdateSmallMaxRows, e.g. one decode step): one warp
 // per instance, the same decisions and sums as launch_update (k_update_small.cu).

@@ -279,6 +279,7 @@ __global__ void __launch_bounds__(32 * kHeadsPerCta, R == 16 ? 2 : 1) cfps_kerne
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int h = blockIdx.x * kHeadsPerCta + wid;
+  grid_dependency_wait();
   if (h >= a.H) return;  // whole warp
   if (MODE == kCfpsMerge && a.Ls) {  // per-instance lengths: no eviction in this instance, nothing to merge
     const int L = a.Ls[h / a.group];
@@ -383,8 +384,7 @@ cudaError_t launch_cfps_m(const CfpsArgs& a, cudaStream_t st) {
   e = cudaFuncSetAttribute(cfps_kernel<D, R, MODE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;
   const int grid = (a.H + kHeadsPerCta - 1) / kHeadsPerCta;
-  cfps_kernel<D, R, MODE><<<grid, 32 * kHeadsPerCta, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(cfps_kernel<D, R, MODE>, static_cast<unsigned>(grid), 32 * kHeadsPerCta, smem, st, a);
 }
 
 template <int D, int R>

@@ -618,8 +618,7 @@ template <int D, int NW, int MT, bool RES>
 cudaError_t launch_fps_dr(const Shape& s, const __nv_bfloat16* q_init, int N, float* cent, double* sums,
                           long long* counts, cudaStream_t st) {
   const size_t smem = fps_layout(N, D, 32 * NW, RES).total;
-  const cudaError_t e = cudaFuncSetAttribute(fps_init_kernel<D, NW, MT, RES>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = allow_smem<fps_init_kernel<D, NW, MT, RES>>(smem);
   if (e != cudaSuccess) return e;
   fps_init_kernel<D, NW, MT, RES><<<s.n_inst, 32 * NW, smem, st>>>(q_init, N, s.nb, cent, sums, counts);
   return cudaGetLastError();

@@ -23,6 +23,7 @@ __global__ void __launch_bounds__(kPlanThreads) ragged_plan_kernel(int n_inst, i
   __shared__ int wsum[kPlanThreads / 32];
   __shared__ int base_sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  grid_dependency_wait();
   if (threadIdx.x == 0) base_sh = 0;
   __syncthreads();
   for (int c0 = 0; c0 < n_inst; c0 += kPlanThreads) {
@@ -52,6 +53,7 @@ __global__ void __launch_bounds__(kPlanThreads) ragged_plan_kernel(int n_inst, i
 
 __global__ void ragged_keep_kernel(int n_inst, int cap, const int* __restrict__ Ls, int budget,
                                    int* __restrict__ kept) {
+  grid_dependency_wait();
   const size_t n = static_cast<size_t>(n_inst) * budget;
   for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<size_t>(gridDim.x) * blockDim.x) {
@@ -67,13 +69,11 @@ __global__ void ragged_keep_kernel(int n_inst, int cap, const int* __restrict__ 
 
 cudaError_t launch_ragged_plan(const Shape& s, const int* Ls, int budget, int* work, int* n_work, int* kept, int* err,
                                cudaStream_t st) {
-  ragged_plan_kernel<<<1, kPlanThreads, 0, st>>>(s.n_inst, s.cap, Ls, budget, work, n_work, err);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_dependent(ragged_plan_kernel, 1, kPlanThreads, 0, st, s.n_inst, s.cap, Ls, budget, work, n_work, err);
   if (e != cudaSuccess) return e;
   const size_t n = static_cast<size_t>(s.n_inst) * budget;
   const int blocks = static_cast<int>(n / 256 + 1 < 4096 ? n / 256 + 1 : 4096);
-  ragged_keep_kernel<<<blocks, 256, 0, st>>>(s.n_inst, s.cap, Ls, budget, kept);
-  return cudaGetLastError();
+  return launch_dependent(ragged_keep_kernel, static_cast<unsigned>(blocks), 256, 0, st, s.n_inst, s.cap, Ls, budget, kept);
 }
 
 }  // namespace bkv

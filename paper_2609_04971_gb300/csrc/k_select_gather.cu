@@ -336,12 +336,9 @@ template <int D>
 cudaError_t launch_sg_d(const Shape& s, float* r, const int* Ls, const int* work, const int* n_work, int L, int budget,
                         __nv_bfloat16* K, __nv_bfloat16* V, int* kept, int* err, cudaStream_t st) {
   const size_t smem = sizeof(uint32_t) * static_cast<size_t>(L);  // every instance has at most L rows
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  if (use_split(s.n_inst, L, budget, sms)) {
-    e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e;
+  if (use_split(s.n_inst, L, budget, device_sms())) {
+    e = allow_smem<select_kernel>(smem);
     if (e != cudaSuccess) return e;
     e = launch_dependent(select_kernel, static_cast<unsigned>(s.n_inst), kSelThreads, smem, st, s, r, L, budget, kept, Ls,
                          work, n_work, err);
@@ -349,7 +346,7 @@ cudaError_t launch_sg_d(const Shape& s, float* r, const int* Ls, const int* work
     return launch_dependent(gather_kernel<D>, static_cast<unsigned>(s.n_inst * (2 * D / 64)), kSgThreads, 0, st, s, r, L,
                             budget, K, V, kept, Ls, work, n_work, err);
   }
-  e = cudaFuncSetAttribute(select_gather_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  e = allow_smem<select_gather_kernel<D>>(smem);
   if (e != cudaSuccess) return e;
   return launch_dependent(select_gather_kernel<D>, static_cast<unsigned>(s.n_inst), kSgThreads, smem, st, s, r, L, budget,
                           K, V, kept, Ls, work, n_work, err);

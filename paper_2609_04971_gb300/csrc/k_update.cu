@@ -379,6 +379,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_dependency_wait();  // the set-up above touched no global memory
   const uint32_t tmem = tmem_base_sh;
   const uint32_t tmem_sums = tmem + kDots * ncols1;  // [kSums][kParts * NBO]
   volatile int* abort_flag = &abort_sh;
@@ -927,11 +928,10 @@ template <int D, int NBO>
 cudaError_t launch_update_dn(const UpdArgs& a, const CUtensorMap& qmap, int grid, cudaStream_t st) {
   using C = UpdCfg<D, NBO>;
   const size_t smem = C::smem_bytes(a.nbp);
-  const cudaError_t e =
-      cudaFuncSetAttribute(update_kernel<D, NBO>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = allow_smem<update_kernel<D, NBO>>(smem);
   if (e != cudaSuccess) return e;
-  update_kernel<D, NBO><<<grid, kUThreads, smem, st>>>(qmap, a, C::stages(a.nbp));
-  const cudaError_t le = cudaGetLastError();
+  const cudaError_t le = launch_dependent(update_kernel<D, NBO>, static_cast<unsigned>(grid), kUThreads, smem, st, qmap, a,
+                                          C::stages(a.nbp));
   if (le != cudaSuccess) return le;
   constexpr int kPer = kFoldThreads / D;
   return launch_dependent(update_fold_kernel<D>, static_cast<unsigned>((a.n_inst + kPer - 1) / kPer), kFoldThreads, 0, st,
@@ -939,23 +939,24 @@ cudaError_t launch_update_dn(const UpdArgs& a, const CUtensorMap& qmap, int grid
 }
 
 int update_grid(int n_inst) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   return n_inst < sms ? n_inst : sms;
 }
 
 }  // namespace
 
-// spill, then the call's sums, then its counts
-size_t update_scratch_words(const Shape& s) {
-  if (s.nb == 0) return 0;
+size_t update_spill_words(const Shape& s) {
+  return s.nb == 0 ? 0 : static_cast<size_t>(update_grid(s.n_inst)) * kSpillSlots * s.nb * s.d;
+}
+
+// the call's sums, then its counts
+size_t update_call_bytes(const Shape& s) {
   const size_t inst = static_cast<size_t>(s.n_inst) * s.nb;
-  return static_cast<size_t>(update_grid(s.n_inst)) * kSpillSlots * s.nb * s.d + inst * s.d + (inst + 1) / 2;
+  return inst * s.d * sizeof(long long) + inst * sizeof(int);
 }
 
 cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows, int n_new,
-                          float* cent, double* sums, long long* counts, int* assign_out, unsigned long long* scratch,
+                          float* cent, double* sums, long long* counts, int* assign_out, unsigned long long* spill, void* call,
                           int* err, cudaStream_t st) {
   UpdArgs a;
   a.n_inst = s.n_inst;
@@ -968,10 +969,9 @@ cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows,
   a.counts = counts;
   a.assign_out = assign_out;
   const int grid = update_grid(s.n_inst);
-  const size_t inst = static_cast<size_t>(s.n_inst) * s.nb;
-  a.spill = scratch;
-  a.call_sum = reinterpret_cast<long long*>(scratch + static_cast<size_t>(grid) * kSpillSlots * s.nb * s.d);
-  a.call_cnt = reinterpret_cast<int*>(a.call_sum + inst * s.d);
+  a.spill = spill;
+  a.call_sum = static_cast<long long*>(call);
+  a.call_cnt = reinterpret_cast<int*>(a.call_sum + static_cast<size_t>(s.n_inst) * s.nb * s.d);
   a.err = err;
   if (s.d == 128)
     return s.nb <= 16 ? launch_update_dn<128, 16>(a, qmap, grid, st) : launch_update_dn<128, 32>(a, qmap, grid, st);

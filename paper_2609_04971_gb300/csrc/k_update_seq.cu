@@ -379,6 +379,7 @@ __global__ void __launch_bounds__(D, (NQ <= 8 ? 6 : 3) * 128 / D) update_seq_ker
     Pm[i] = __int_as_float(__double2hiint(v));
   };
 
+  grid_dependency_wait();
   for (int e = blockIdx.x; e < a.n_inst; e += gridDim.x) {
     const size_t cbase = static_cast<size_t>(e) * nb * D;
     // ---- this warp's columns of the instance's state (4 beacons' loads in flight per lane); the sums
@@ -672,8 +673,7 @@ cudaError_t launch_seq_dq(const SeqArgs& a, int sms, cudaStream_t st) {
   if (per_sm < 1) return cudaErrorInvalidValue;
   const long long slots = 1ll * per_sm * sms;
   const int grid = static_cast<int>(a.n_inst < slots ? a.n_inst : slots);
-  update_seq_kernel<D, NQ><<<grid, D, lay.total, st>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(update_seq_kernel<D, NQ>, static_cast<unsigned>(grid), D, lay.total, st, a);
 }
 
 template <int D>
@@ -692,10 +692,8 @@ cudaError_t launch_update_seq(const Shape& s, const __nv_bfloat16* q_steps, int 
   if (s.G > kUpdateSmallMaxRows || s.nb > kMaxBeacons) return cudaErrorInvalidValue;
   int lg = 0;
   while ((32 >> (lg + 1)) >= s.nb && lg < 3) ++lg;  // 2^lg lanes per row, 2^lg * nb <= 32
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
+  const int sms = device_sms();
+  if (sms < 1) return cudaErrorInvalidDevice;
   SeqArgs a{s.n_inst, s.G, s.nb, n_steps, lg, q_steps, cent, sums, counts, assign_out};
   return s.d == 128 ? launch_seq_d<128>(a, sms, st) : launch_seq_d<64>(a, sms, st);
 }

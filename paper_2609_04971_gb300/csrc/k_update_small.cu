@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(32 * SmallLayout<D, NQ>::kWarps, NQ <= 8 ? 4 :
   extern __shared__ __align__(16) float small_sh[];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int e = blockIdx.x * Lay::kWarps + w;
+  grid_dependency_wait();
   if (e >= a.n_inst) return;  // whole warp
   const int nb = a.nb, nq = a.nq;
   float* qs = small_sh + static_cast<size_t>(w) * Lay::kPerWarp + Lay::kQs;
@@ -321,11 +322,10 @@ template <int D, int NQ>
 cudaError_t launch_small_dq(const SmallArgs& a, cudaStream_t st) {
   using Lay = SmallLayout<D, NQ>;
   const size_t smem = sizeof(float) * Lay::kWarps * Lay::kPerWarp;
-  cudaError_t e = cudaFuncSetAttribute(update_small_kernel<D, NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  const cudaError_t e = allow_smem<update_small_kernel<D, NQ>>(smem);
   if (e != cudaSuccess) return e;
-  update_small_kernel<D, NQ><<<(a.n_inst + Lay::kWarps - 1) / Lay::kWarps, 32 * Lay::kWarps, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(update_small_kernel<D, NQ>, static_cast<unsigned>((a.n_inst + Lay::kWarps - 1) / Lay::kWarps),
+                          32 * Lay::kWarps, smem, st, a);
 }
 
 template <int D>
