@@ -33,10 +33,11 @@
 // centroids), never below -11, so that what the operands hold is exact in fixed
 // point with 40 fractional bits; the result does not depend on it.
 //
-// The call's sums (int64, 40 fractional bits) and counts go to scratch, from where
-// update_fold_kernel adds them once to the fp64 running sums, correctly rounded
-// and without fp64 arithmetic (slow on this part), and forms c = fp32(sum / count)
-// to within one fp32 ulp from double-float arithmetic on the sum's bits.
+// The call's sums (int64, 40 fractional bits) and counts go to scratch.  After its
+// last tile the CTA adds them once to the fp64 running sums of its instances,
+// correctly rounded and without fp64 arithmetic (slow on this part), and forms
+// c = fp32(sum / count) to within one fp32 ulp from double-float arithmetic on the
+// sum's bits.
 //
 // Warp roles (23 warps): warp 0 TMA producer; warp 1 TMEM allocation and the
 // screening MMAs; warp 2 the sums' MMAs; warps 3..10 two groups of four that
@@ -51,7 +52,7 @@
 // so loops are kept rolled and rare paths small (re-decisions and spilled elements,
 // three tiles in ten, still cost a fifth of the time).  Sums formed in fp32 parts
 // by CUDA cores from rows sorted by beacon took about 14 K warp instructions per
-// tile.  With the fold kernel: 4608 instances x 512 queries of 128, 8 beacons: 393
+// tile.  With the fold: 4608 instances x 512 queries of 128, 8 beacons: 393
 // us, now 255 (95 at the copy rate); 8192 instances, 16 beacons: 815 us, now 485
 // (206).
 #include "bkv_device.cuh"
@@ -91,7 +92,7 @@ struct UpdArgs {
   long long* counts;
   int* assign_out;
   unsigned long long* spill;  // [grid][kSpillSlots][nb][D], zero between instances
-  long long* call_sum;        // [n_inst][nb][D]: this call's sums, units of 2^-40, for the fold kernel
+  long long* call_sum;        // [n_inst][nb][D]: this call's sums, units of 2^-40
   int* call_cnt;              // [n_inst][nb]: queries assigned
   int* err;
 };
@@ -741,7 +742,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
       }
       if (T > kFlush) named_barrier(1, 256);  // what another warp passed on (d = 64) is there
 
-      // ---- this instance's sums of the call, for the fold kernel
+      // ---- this instance's sums of the call, for the fold at the end
       const int add = lane < nb ? add_cnt[slot][lane] : 0;
       const int shift = static_cast<signed char>(exp_sh[slot] & 0xff) + 40 - (kSmallBits + 7);  // to units of 2^-40
       const bool spilled = spilled_sh[slot] != 0;
@@ -866,61 +867,46 @@ __global__ void __launch_bounds__(kUThreads, 1)
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
-}
+  if (*abort_flag) return;  // a wait gave up: some sums are missing
 
-// The call's sums into the running state: thread = (instance, column), its beacons in fours.  A kernel of
-// its own: as a role of update_kernel its instructions kept the other roles waiting for theirs (4608
-// instances of 8 beacons 298 -> 270 us, 8192 of 16 537 -> 516 us, this kernel included).  What bounds it:
-// 28 bytes and about 130 instructions per cell.
-constexpr int kFoldThreads = 128;
-template <int D>
-__global__ void __launch_bounds__(kFoldThreads) update_fold_kernel(int n_inst, int nb, const long long* __restrict__ call_sum,
-                                                                   const int* __restrict__ call_cnt, float* cent,
-                                                                   double* sums, long long* counts) {
-  constexpr int kPer = kFoldThreads / D;  // instances per block
-  constexpr int kChunk = 4;
-  __shared__ DF rcp[kPer][kMaxBeacons];
-  __shared__ int added[kPer][kMaxBeacons];
-  const int sub = threadIdx.x / D, col = threadIdx.x % D;
-  const int e = blockIdx.x * kPer + sub;
-  grid_dependency_wait();
-  if (e < n_inst && col < nb) {
-    const size_t i = static_cast<size_t>(e) * nb + col;
-    const int add = call_cnt[i];
-    added[sub][col] = add;
-    if (add > 0) {
-      const long long n = counts[i] + add;
-      counts[i] = n;
-      rcp[sub][col] = count_reciprocal(n);
+  // ---- this CTA's instances: the call's sums into the running state, a warp per (instance, beacon).  After
+  // the tiles, not as a role beside them: there its instructions kept the other roles waiting for theirs
+  // (4608 instances of 8 beacons 298 -> 255 us, 8192 of 16 537 -> 485 us by taking it out).  What bounds it:
+  // 28 bytes and about 130 instructions per cell.
+  constexpr int kCells = D / 32;
+  for (int unit = warp; unit < n_my * nb; unit += kUThreads / 32) {
+    const int i = unit / nb, b = unit - i * nb;
+    const size_t row = (static_cast<size_t>(blockIdx.x) + static_cast<size_t>(i) * gridDim.x) * nb + b;
+    const int add = __ldcg(a.call_cnt + row);
+    if (add == 0) continue;  // warp-uniform
+    const size_t base = row * D + lane;
+    double s_old[kCells], s_new[kCells];
+    long long f[kCells];
+    float c_new[kCells];
+#pragma unroll
+    for (int k = 0; k < kCells; ++k) {
+      s_old[k] = a.sums[base + 32 * k];
+      f[k] = __ldcg(a.call_sum + base + 32 * k);
     }
-  }
-  __syncthreads();
-  if (e >= n_inst) return;
-  const size_t base = static_cast<size_t>(e) * nb * D + col;
-  for (int b0 = 0; b0 < nb; b0 += kChunk) {
-    double s_old[kChunk], s_new[kChunk];
-    long long f[kChunk];
-    float c_new[kChunk];
-    bool mine[kChunk], ok[kChunk];
+    const long long n = a.counts[row] + add;
+    const DF rcp = count_reciprocal(n);
+    bool plain = true;
 #pragma unroll
-    for (int u = 0; u < kChunk; ++u) {
-      mine[u] = b0 + u < nb && added[sub][b0 + u < nb ? b0 + u : 0] > 0;
-      s_old[u] = mine[u] ? sums[base + static_cast<size_t>(b0 + u) * D] : 1.0;
-      f[u] = mine[u] ? __ldcs(call_sum + base + static_cast<size_t>(b0 + u) * D) : 0;
-    }
+    for (int k = 0; k < kCells; ++k) plain &= fold_and_centroid(s_old[k], f[k], rcp, s_new[k], c_new[k]);
+    if (!plain) {  // a sum off the 2^-40 grid, past 2^22 or zero
 #pragma unroll
-    for (int u = 0; u < kChunk; ++u)
-      ok[u] = fold_and_centroid(s_old[u], f[u], rcp[sub][b0 + u < nb ? b0 + u : 0], s_new[u], c_new[u]);
-#pragma unroll
-    for (int u = 0; u < kChunk; ++u)
-      if (mine[u]) {
-        if (!ok[u]) {  // a sum off the 2^-40 grid, past 2^22 or zero
-          s_new[u] = fold_sum(s_old[u], f[u]);
-          c_new[u] = centroid_value(s_new[u], rcp[sub][b0 + u]);
-        }
-        sums[base + static_cast<size_t>(b0 + u) * D] = s_new[u];
-        cent[base + static_cast<size_t>(b0 + u) * D] = c_new[u];
+      for (int k = 0; k < kCells; ++k) {
+        s_new[k] = fold_sum(s_old[k], f[k]);
+        c_new[k] = centroid_value(s_new[k], rcp);
       }
+    }
+#pragma unroll
+    for (int k = 0; k < kCells; ++k) {
+      a.sums[base + 32 * k] = s_new[k];
+      a.cent[base + 32 * k] = c_new[k];
+    }
+    __syncwarp();  // every lane has read the count
+    if (lane == 0) a.counts[row] = n;
   }
 }
 
@@ -930,12 +916,8 @@ cudaError_t launch_update_dn(const UpdArgs& a, const CUtensorMap& qmap, int grid
   const size_t smem = C::smem_bytes(a.nbp);
   const cudaError_t e = allow_smem<update_kernel<D, NBO>>(smem);
   if (e != cudaSuccess) return e;
-  const cudaError_t le = launch_dependent(update_kernel<D, NBO>, static_cast<unsigned>(grid), kUThreads, smem, st, qmap, a,
-                                          C::stages(a.nbp));
-  if (le != cudaSuccess) return le;
-  constexpr int kPer = kFoldThreads / D;
-  return launch_dependent(update_fold_kernel<D>, static_cast<unsigned>((a.n_inst + kPer - 1) / kPer), kFoldThreads, 0, st,
-                          a.n_inst, a.nb, a.call_sum, a.call_cnt, a.cent, a.sums, a.counts);
+  return launch_dependent(update_kernel<D, NBO>, static_cast<unsigned>(grid), kUThreads, smem, st, qmap, a,
+                          C::stages(a.nbp));
 }
 
 int update_grid(int n_inst) {
