@@ -27,7 +27,7 @@
 // |x| >= 2^(E-20)), whose sums over 128 rows stay below 2^24 grid steps, so the
 // fp32 accumulator never rounds.  The two sums of a (column, beacon) cell are
 // integers, added up over the tiles in two registers.  The few elements outside
-// [2^(E-20), 2^E) (one in five tiles of normal data) are zeroed in the operands
+// [2^(E-20), 2^E) (one in ten tiles of normal data) are zeroed in the operands
 // and added as a list (past 32 per instance through a global array of this CTA).
 // E comes from the largest |q| this CTA has seen (before that from the
 // centroids), never below -11, so that what the operands hold is exact in fixed
@@ -52,9 +52,9 @@
 // so loops are kept rolled and rare paths small (re-decisions and spilled elements,
 // three tiles in ten, still cost a fifth of the time).  Sums formed in fp32 parts
 // by CUDA cores from rows sorted by beacon took about 14 K warp instructions per
-// tile.  With the fold: 4608 instances x 512 queries of 128, 8 beacons: 393
-// us, now 255 (95 at the copy rate); 8192 instances, 16 beacons: 815 us, now 485
-// (206).
+// tile.  With the fold (in a launch of its own: 255 and 485 us): 4608 instances x 512 queries of 128, 8 beacons: 393
+// us, now 242 (95 at the copy rate); 8192 instances, 16 beacons: 815 us, now 476
+// (178).
 #include "bkv_device.cuh"
 #include "bkv_internal.h"
 #include "k_update_math.cuh"

@@ -220,6 +220,7 @@ __device__ __forceinline__ double fold_sum(double s, long long acc) {
 // fold_sum for warps that have the fp64 pipe to themselves: below 2^53, acc * 2^-40 is exact in
 // fp64 and one fp64 addition rounds the sum once, so the result is fold_sum's, without its integer
 // instructions; larger sums take fold_sum (which rounds once where the fp64 route would round twice).
+// No kernel takes this form now; tests/cuda/fold_check.cu compares it with fold_sum.
 __device__ __forceinline__ double fold_sum_fp64(double s, long long acc) {
   const long long lim = 1LL << 53;
   if (acc > -lim && acc < lim) return acc == 0 ? s : __dadd_rn(s, fixed40_to_double(acc));
