@@ -59,7 +59,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 
 // Waits until the kernels that this one depends on have completed and their writes are visible.  A
 // kernel launched by launch_dependent starts before that, so every thread that touches global memory
-// calls it first; without that launch attribute it returns at once.
+// calls it first; without that launch attribute it returns at once.  Such a kernel's pointers are not
+// __restrict__ and its loads not read-only ones (.nc, __ldg): what the kernel before writes is not
+// constant for this one, and a pointer declared unaliased may be read before the wait.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ------------------------------------------------------------------ mbarrier

@@ -97,7 +97,8 @@ struct RawWords {
   static constexpr int n = (D / 64) * (F32 ? 2 : 1);
 };
 
-// Issues the global loads of cnt <= kChunk rows: lane l takes elements 2l, 2l+1 (+ 64 when d = 128).
+// Issues the global loads of cnt <= kChunk rows: lane l takes elements 2l, 2l+1 (+ 64 when d = 128).  Ordinary
+// loads: the launch before may still be writing the rows when this kernel starts (see grid_dependency_wait).
 template <int D, bool F32, typename Src>
 __device__ __forceinline__ void load_rows(uint32_t (&raw)[kChunk][RawWords<D, F32>::n], bool (&f32)[kChunk], int cnt,
                                           Src src) {
@@ -115,7 +116,7 @@ __device__ __forceinline__ void load_rows(uint32_t (&raw)[kChunk][RawWords<D, F3
         if (rs.f32) {
 #pragma unroll
           for (int h = 0; h < D / 64; ++h)
-            asm volatile("ld.global.nc.v2.u32 {%0,%1}, [%2];"
+            asm volatile("ld.global.v2.u32 {%0,%1}, [%2];"
                          : "=r"(raw[u][2 * h]), "=r"(raw[u][2 * h + 1])
                          : "l"(base + h * 256 + lane * 8));
           continue;
@@ -123,7 +124,7 @@ __device__ __forceinline__ void load_rows(uint32_t (&raw)[kChunk][RawWords<D, F3
       }
 #pragma unroll
       for (int h = 0; h < D / 64; ++h)
-        asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(raw[u][h]) : "l"(base + h * 128 + lane * 4));
+        asm volatile("ld.global.u32 %0, [%1];" : "=r"(raw[u][h]) : "l"(base + h * 128 + lane * 4));
     }
   }
 }

@@ -55,14 +55,11 @@ __device__ __forceinline__ __nv_bfloat16 rot_fast(float xa, float xb, float c32,
 
 // work / n_work (per-instance lengths): block w builds instance work[w] when w < *n_work; rope_row: the
 // distance between two batch rows' rotary tables (0: one table for every instance).
-__global__ void __launch_bounds__(kQobsThreads) qobs_kernel(Shape s, const __nv_bfloat16* __restrict__ q_recent,
-                                                             const float* __restrict__ cent,
-                                                             const long long* __restrict__ counts,
-                                                             const double2* __restrict__ rope_all, size_t rope_row,
-                                                             int rotate, const int* __restrict__ work,
-                                                             const int* __restrict__ n_work,
-                                                             __nv_bfloat16* __restrict__ qobs,
-                                                             uint32_t* __restrict__ valid, int* err) {
+__global__ void __launch_bounds__(kQobsThreads) qobs_kernel(Shape s, const __nv_bfloat16* q_recent, const float* cent,
+                                                             const long long* counts, const double2* rope_all,
+                                                             size_t rope_row, int rotate, const int* work,
+                                                             const int* n_work, __nv_bfloat16* qobs, uint32_t* valid,
+                                                             int* err) {
   int e = blockIdx.x;
   grid_dependency_wait();
   if (work) {

@@ -17,9 +17,8 @@ namespace {
 
 constexpr int kPlanThreads = 1024;
 
-__global__ void __launch_bounds__(kPlanThreads) ragged_plan_kernel(int n_inst, int cap, const int* __restrict__ Ls,
-                                                                    int budget, int* __restrict__ work,
-                                                                    int* __restrict__ n_work, int* err) {
+__global__ void __launch_bounds__(kPlanThreads) ragged_plan_kernel(int n_inst, int cap, const int* Ls,
+                                                                    int budget, int* work, int* n_work, int* err) {
   __shared__ int wsum[kPlanThreads / 32];
   __shared__ int base_sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -51,8 +50,7 @@ __global__ void __launch_bounds__(kPlanThreads) ragged_plan_kernel(int n_inst, i
   if (threadIdx.x == 0) *n_work = base_sh;
 }
 
-__global__ void ragged_keep_kernel(int n_inst, int cap, const int* __restrict__ Ls, int budget,
-                                   int* __restrict__ kept) {
+__global__ void ragged_keep_kernel(int n_inst, int cap, const int* Ls, int budget, int* kept) {
   grid_dependency_wait();
   const size_t n = static_cast<size_t>(n_inst) * budget;
   for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;

@@ -161,11 +161,12 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity, int* 
   mbar_wait(bar, parity, &never, err, kDevTimeoutDrain);
 }
 
-// Read-only global load emitted exactly here (the compiler may not sink it
-// towards its first use, where its latency behind the K stream would show).
-__device__ __forceinline__ uint32_t ld_nc_u32(const uint32_t* p) {
+// Global load emitted exactly here (the compiler may not sink it towards its first
+// use, where its latency behind the K stream would show).  Not a read-only (.nc)
+// load: the launch before writes the words (see grid_dependency_wait).
+__device__ __forceinline__ uint32_t ld_here_u32(const uint32_t* p) {
   uint32_t v;
-  asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
 }
 
@@ -594,13 +595,13 @@ __global__ void __launch_bounds__(kScThreads, 1)
     // is the valid count of the mean form).
     const int vw = COMBINE ? ((col0 >> 5) + (te >> 5)) & 3 : te >> 5;  // this thread's valid word
     int e_next = n_my > 0 ? item_inst(a, cluster_id, s.n_inst) : 0;
-    uint32_t vnext = (te < 128 && n_my > 0) ? ld_nc_u32(&a.valid[e_next * 4 + vw]) : 0u;
+    uint32_t vnext = (te < 128 && n_my > 0) ? ld_here_u32(&a.valid[e_next * 4 + vw]) : 0u;
     for (int i = 0; i < n_my; ++i) {
       const int e = e_next;
       const uint32_t vword = vnext;
       if (i + 1 < n_my) {
         e_next = item_inst(a, cluster_id + (i + 1) * n_clusters, s.n_inst);
-        if (te < 128) vnext = ld_nc_u32(&a.valid[e_next * 4 + vw]);
+        if (te < 128) vnext = ld_here_u32(&a.valid[e_next * 4 + vw]);
       }
       const int L_e = inst_len(a, e);
       const Geom gm = inst_geom(L_e, crank, csize, ring);

@@ -183,11 +183,10 @@ __device__ __forceinline__ bool block_instance(const Shape& s, int w, const int*
 }
 
 template <int D>
-__global__ void __launch_bounds__(kSgThreads) select_gather_kernel(Shape s, const float* __restrict__ r, int L,
-                                                                    int budget, __nv_bfloat16* K, __nv_bfloat16* V,
-                                                                    int* kept, const int* __restrict__ Ls,
-                                                                    const int* __restrict__ work,
-                                                                    const int* __restrict__ n_work, int* err) {
+__global__ void __launch_bounds__(kSgThreads) select_gather_kernel(Shape s, const float* r, int L, int budget,
+                                                                    __nv_bfloat16* K, __nv_bfloat16* V, int* kept,
+                                                                    const int* Ls, const int* work, const int* n_work,
+                                                                    int* err) {
   extern __shared__ __align__(16) uint32_t keys[];  // [L]
   int e, first;
   if (!block_instance(s, blockIdx.x, Ls, work, n_work, e, L, err)) return;  // whole block
@@ -241,8 +240,8 @@ __global__ void __launch_bounds__(kSgThreads) select_gather_kernel(Shape s, cons
 // ---- split form
 // Selection only.  The instance's first score, read by now, receives the first evicted row.
 __global__ void __launch_bounds__(kSelThreads) select_kernel(Shape s, float* r, int L, int budget, int* kept,
-                                                             const int* __restrict__ Ls, const int* __restrict__ work,
-                                                             const int* __restrict__ n_work, int* err) {
+                                                             const int* Ls, const int* work, const int* n_work,
+                                                             int* err) {
   extern __shared__ __align__(16) uint32_t keys[];  // [L]
   int e, first;
   if (!block_instance(s, blockIdx.x, Ls, work, n_work, e, L, err)) return;  // whole block
@@ -255,11 +254,10 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(Shape s, float* r, 
 // in-place rule (see the file comment) holds slice by slice.  A chunk is 256 rows, eight per thread; its
 // kept indices pass through shared memory two chunks ahead.
 template <int D>
-__global__ void __launch_bounds__(kSgThreads, 3) gather_kernel(Shape s, const float* __restrict__ r, int L, int budget,
-                                                            __nv_bfloat16* K, __nv_bfloat16* V,
-                                                            const int* __restrict__ kept, const int* __restrict__ Ls,
-                                                            const int* __restrict__ work,
-                                                            const int* __restrict__ n_work, int* err) {
+__global__ void __launch_bounds__(kSgThreads, 3) gather_kernel(Shape s, const float* r, int L, int budget,
+                                                            __nv_bfloat16* K, __nv_bfloat16* V, const int* kept,
+                                                            const int* Ls, const int* work, const int* n_work,
+                                                            int* err) {
   constexpr int kSlices = 2 * D / 64;     // 128-byte slices of K, then of V
   constexpr int kVpr = D * 2 / 16;        // 16-byte vectors per row of one tensor
   constexpr int kPer = 8;
