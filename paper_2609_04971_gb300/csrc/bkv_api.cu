@@ -27,7 +27,9 @@ struct bkv_ctx {
   float* cent = nullptr;
   double* sums = nullptr;
   long long* counts = nullptr;
-  unsigned long long* spill = nullptr;  // batched update: zero between calls (update_spill_words)
+  int update_grid = 0;                  // batched update: CTAs of a launch
+  unsigned long long* spill = nullptr;  // [n_spill], zero between batched updates (update_spill_words)
+  size_t n_spill = 0;
   bool state_ready = false;
   // Continual FPS (BKV_F_CONTINUAL_FPS): per-query-head buffers; cent / counts then hold each
   // compress's beacons ([n_inst][G * n_beacons] rows, count 1 or 0) for the scoring-query build
@@ -274,11 +276,14 @@ int bkv_create(const bkv_config* cfg, void* stream, bkv_ctx** out) {
   const size_t nh = static_cast<size_t>(c->n_heads);
   // the compress's scores; a batched update's sums use the same memory (neither outlives its call)
   const size_t n_rscore = std::max(ni * s.cap, c->cfps ? 0 : (bkv::update_call_bytes(s) + 3) / 4);
-  const size_t n_spill = c->cfps ? 0 : bkv::update_spill_words(s);
+  // a batched update's CTAs, fixed here with the scratch they use
+  const int sms = bkv::device_sms();
+  c->update_grid = std::min(s.n_inst, sms);
+  c->n_spill = c->cfps ? 0 : bkv::update_spill_words(s, c->update_grid);
   if ((e = dmalloc(&c->cent, ni * s.nb * s.d)) != cudaSuccess ||
       (e = dmalloc(&c->sums, c->cfps ? 0 : ni * s.nb * s.d)) != cudaSuccess ||
       (e = dmalloc(&c->counts, ni * s.nb)) != cudaSuccess ||
-      (e = dmalloc(&c->spill, n_spill)) != cudaSuccess ||
+      (e = dmalloc(&c->spill, c->n_spill)) != cudaSuccess ||
       (e = dmalloc(&c->cbuf, nh * c->b_max * s.d)) != cudaSuccess ||
       (e = dmalloc(&c->csize, nh)) != cudaSuccess ||
       (e = dmalloc(&c->qobs, ni * s.n_obs_pad * s.d)) != cudaSuccess ||
@@ -287,7 +292,7 @@ int bkv_create(const bkv_config* cfg, void* stream, bkv_ctx** out) {
       (e = dmalloc(&c->rope, static_cast<size_t>(s.W + 1) * (s.d / 2) * 3 / 2 + 1)) != cudaSuccess ||
       (e = dmalloc(&c->work, ni)) != cudaSuccess || (e = dmalloc(&c->n_work, 1)) != cudaSuccess ||
       (e = dmalloc(&c->rag, c->rag_bytes)) != cudaSuccess ||
-      (e = dmalloc(&c->err, 1)) != cudaSuccess) {
+      (e = dmalloc(&c->err, 1)) != cudaSuccess || (e = sms > 0 ? cudaSuccess : cudaErrorInvalidDevice) != cudaSuccess) {
     const int code = (e == cudaErrorMemoryAllocation) ? BKV_ENOMEM : BKV_ECUDA;
     cudaGetLastError();
     free_all(c);
@@ -296,7 +301,7 @@ int bkv_create(const bkv_config* cfg, void* stream, bkv_ctx** out) {
   }
   if ((e = cudaMemsetAsync(c->cent, 0, sizeof(float) * ni * s.nb * s.d + 0, c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->sums, 0, sizeof(double) * (c->cfps ? 1 : ni * s.nb * s.d), c->stream)) != cudaSuccess ||
-      (e = cudaMemsetAsync(c->spill, 0, sizeof(unsigned long long) * (n_spill ? n_spill : 1), c->stream)) != cudaSuccess ||
+      (e = cudaMemsetAsync(c->spill, 0, sizeof(unsigned long long) * c->n_spill, c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->csize, 0, sizeof(int) * (nh ? nh : 1), c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->counts, 0, sizeof(long long) * ni * s.nb, c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->err, 0, sizeof(int), c->stream)) != cudaSuccess) {
@@ -427,8 +432,8 @@ int bkv_update_beacons(bkv_ctx* ctx, const void* q_new, int32_t n_new, int32_t* 
   const int rc = encode_rows(ctx, &qmap, q_new, q_rows, s.d, static_cast<uint32_t>(box_rows));
   if (rc != BKV_OK) return rc;
   ProfScope ps(ctx, BKV_K_UPDATE);
-  cudaError_t e = bkv::launch_update(s, qmap, static_cast<int>(box_rows), n_new,
-                                     ctx->cent, ctx->sums, ctx->counts, assign_out, ctx->spill, ctx->rscore, ctx->err, ctx->stream);
+  cudaError_t e = bkv::launch_update(s, qmap, static_cast<int>(box_rows), n_new, ctx->update_grid, ctx->cent, ctx->sums,
+                                     ctx->counts, assign_out, ctx->spill, ctx->rscore, ctx->err, ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "update launch");
   return BKV_OK;
 }
@@ -802,9 +807,11 @@ int bkv_sync(bkv_ctx* ctx) {
   if ((e = cudaMemcpy(&h, ctx->err, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess)
     return cuda_fail(ctx, e, "error word read");
   if (h != 0) {
-    cudaMemset(ctx->err, 0, sizeof(int));
-    // an update that gave up a wait may have left its spill words set
-    if (!ctx->cfps) cudaMemset(ctx->spill, 0, sizeof(unsigned long long) * bkv::update_spill_words(ctx->shape));
+    // On the context's stream, so that the next call's kernels find both cleared.  An update that gave up a
+    // wait may have left its spill words set, and the word keeps only the first error: any of them clears.
+    if ((e = cudaMemsetAsync(ctx->err, 0, sizeof(int), ctx->stream)) != cudaSuccess ||
+        (e = cudaMemsetAsync(ctx->spill, 0, sizeof(unsigned long long) * ctx->n_spill, ctx->stream)) != cudaSuccess)
+      return cuda_fail(ctx, e, "error word clear");
     if (h == bkv::kDevBadLength)
       return fail(ctx, BKV_EINVAL, "a per-instance cache length was outside 1..capacity; that instance was left untouched");
     if (h == bkv::kDevBounds)

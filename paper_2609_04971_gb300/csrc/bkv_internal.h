@@ -112,11 +112,12 @@ cudaError_t launch_fps_init(const Shape& s, const __nv_bfloat16* q_init, int n_i
                             long long* counts, cudaStream_t st);
 
 // qmap: the new queries as [n_inst * G * n_new][d] bf16 in boxes of
-// [box_rows][64] (128-byte swizzle), box_rows = min(128, rows); spill: update_spill_words(s) zeros, which
-// the call leaves zero; call: update_call_bytes(s) of scratch; err: device error word.
-size_t update_spill_words(const Shape& s);
+// [box_rows][64] (128-byte swizzle), box_rows = min(128, rows); grid: CTAs (at most one per SM and one per
+// instance); spill: update_spill_words(s, grid) zeros, which the call leaves zero; call: update_call_bytes(s)
+// of scratch; err: device error word.
+size_t update_spill_words(const Shape& s, int grid);
 size_t update_call_bytes(const Shape& s);
-cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows, int n_new, float* cent,
+cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows, int n_new, int grid, float* cent,
                           double* sums, long long* counts, int* assign_out, unsigned long long* spill, void* call, int* err,
                           cudaStream_t st);
 // A few queries per instance (G * n_new <= kUpdateSmallMaxRows, e.g. one decode step): one warp

@@ -920,15 +920,10 @@ cudaError_t launch_update_dn(const UpdArgs& a, const CUtensorMap& qmap, int grid
                           C::stages(a.nbp));
 }
 
-int update_grid(int n_inst) {
-  const int sms = device_sms();
-  return n_inst < sms ? n_inst : sms;
-}
-
 }  // namespace
 
-size_t update_spill_words(const Shape& s) {
-  return s.nb == 0 ? 0 : static_cast<size_t>(update_grid(s.n_inst)) * kSpillSlots * s.nb * s.d;
+size_t update_spill_words(const Shape& s, int grid) {
+  return static_cast<size_t>(grid) * kSpillSlots * s.nb * s.d;
 }
 
 // the call's sums, then its counts
@@ -937,9 +932,9 @@ size_t update_call_bytes(const Shape& s) {
   return inst * s.d * sizeof(long long) + inst * sizeof(int);
 }
 
-cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows, int n_new,
-                          float* cent, double* sums, long long* counts, int* assign_out, unsigned long long* spill, void* call,
-                          int* err, cudaStream_t st) {
+cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows, int n_new, int grid, float* cent,
+                          double* sums, long long* counts, int* assign_out, unsigned long long* spill, void* call, int* err,
+                          cudaStream_t st) {
   UpdArgs a;
   a.n_inst = s.n_inst;
   a.nq = s.G * n_new;
@@ -950,7 +945,6 @@ cudaError_t launch_update(const Shape& s, const CUtensorMap& qmap, int box_rows,
   a.sums = sums;
   a.counts = counts;
   a.assign_out = assign_out;
-  const int grid = update_grid(s.n_inst);
   a.spill = spill;
   a.call_sum = static_cast<long long*>(call);
   a.call_cnt = reinterpret_cast<int*>(a.call_sum + static_cast<size_t>(s.n_inst) * s.nb * s.d);
