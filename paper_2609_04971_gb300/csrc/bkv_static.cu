@@ -140,8 +140,8 @@ extern "C" int bkv_compress_static(const bkv_config* cfg, const float* centroids
   // the scoring inputs matter only when rows are evicted; checked before anything is enqueued
   if (L > budget && s.W > 0 && (!q_recent || !aligned(q_recent, 16) || !recent_pos))
     return bad("q_recent (16-byte aligned) and recent_pos are required when window > 0");
-  if (L > budget && s.nb > 0 && (!centroids || !counts || !aligned(centroids, 4) || !aligned(counts, 8)))
-    return bad("centroids and counts are required when n_beacons > 0");
+  if (L > budget && s.nb > 0 && (!centroids || !counts || !aligned(centroids, 16) || !aligned(counts, 8)))
+    return bad("centroids (16-byte aligned) and counts (8-byte aligned) are required when n_beacons > 0");
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e;
