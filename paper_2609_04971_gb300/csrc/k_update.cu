@@ -11,14 +11,16 @@
 // bf16(c / |c| - c_hi), so dot_b = D1[:, b] + D1[:, nbp + b] carries the
 // unit-centroid dot to about 2^-16 |q| (bf16 x bf16 products are exact, the
 // accumulation is fp32).  When best and second-best dots differ by at most
-// 7e-5 |q| (kScreenMargin; the bound is 4.2e-5 |q|, and |q| is taken a few
-// percent too large), the query is re-decided exactly: the beacon maximising
-// (q . c_b) / |c_b| in double-float arithmetic (exact products, TwoSum
-// accumulation, 1 / |c_b| from a double-float sum of squares and one Newton
-// step, to about 2^-44 relative), which agrees with the cosine (q . c_b) /
-// (|q| |c_b|) evaluated in fp64 except at ties below ~1e-12 (the lowest beacon
-// wins ties).  Only beacons screened within 1.4e-4 |q| of the best enter that
-// comparison.  Zero queries and instances without a valid beacon give -1.
+// 7e-5 |q| (kScreenMargin; the bound is 4.2e-5 |q|), the query is re-decided
+// exactly: the beacon maximising (q . c_b) / |c_b| in double-float arithmetic
+// (exact products, TwoSum accumulation, 1 / |c_b| from a double-float sum of
+// squares and one Newton step, to about 2^-44 relative), which agrees with the
+// cosine (q . c_b) / (|q| |c_b|) evaluated in fp64 except at ties below ~1e-12
+// (the lowest beacon wins ties).  Only beacons screened within 1.4e-4 |q| of the
+// best enter that comparison.  |q| is formed, in fp32, only where the larger
+// sqrt(d) max|q_i| (exact: a packed maximum) does not rule a re-decision out (8192
+// instances of 512 queries, call and state read: 534 us, with an fp32 sum for
+// every query 574).  Zero queries and instances without a valid beacon give -1.
 //
 // Sums: Q^T x A, where A is the tile's one-hot assignment matrix (128 queries x
 // beacons), exact: an element x with |x| < 2^E (E chosen per instance) goes
@@ -29,7 +31,7 @@
 // integers, added up over the tiles in two registers.  The few elements outside
 // [2^(E-20), 2^E) (one in ten tiles of normal data) are zeroed in the operands
 // and added as a list (past 32 per instance through a global array of this CTA).
-// E comes from the largest |q| this CTA has seen (before that from the
+// E comes from the largest element this CTA has seen (before that from the
 // centroids), never below -11, so that what the operands hold is exact in fixed
 // point with 40 fractional bits; the result does not depend on it.
 //
@@ -80,6 +82,8 @@ constexpr size_t kUSmemBudget = 220 * 1024;
 // A screened dot is within 2^-18 |q| (the hi / lo split) + 136 * 2^-23 |q| (17 additions in each of eight
 // K = 16 steps) + 2^-21 |q| (1 / |c|) of the exact one, so a difference of two within 4.2e-5 |q|.
 constexpr float kScreenMargin = 7e-5f;
+// Queries whose largest element is in this range have a squared norm that fp32 holds (1e-30 < |q|^2 < 1e30).
+constexpr float kTameLo = 1.7763568394002505e-15f, kTameHi = 70368744177664.f;  // 2^-49, 2^46
 constexpr int kMinE = -11, kMaxE = 14;
 constexpr int kLargeBits = 10;              // octaves below 2^E that the tile itself holds
 constexpr int kSmallBits = 20;              // octaves below 2^E that the operands hold
@@ -158,12 +162,6 @@ __device__ __forceinline__ void st_shared_v4_if(uint32_t cond, void* p, uint32_t
       : "memory");
 }
 
-__device__ __forceinline__ float sqrt_approx(float x) {
-  float y;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // bf16 bits of 2^k, in both halves of a word.
 __device__ __forceinline__ uint32_t pow2_bf16x2(int k) {
   const uint32_t b = static_cast<uint32_t>(k + 127) << 7;
@@ -239,6 +237,23 @@ __device__ __noinline__ int refine_row(const unsigned char* raw, const unsigned 
   return best_b;
 }
 
+// fp32 squared norm of this thread's query: a chunk's elements sit in the raw tile or, where that holds 0, in
+// the second one.  Out of line and rolled: rare.
+template <int D>
+__device__ __noinline__ float row_norm2(const unsigned char* raw_row, const unsigned char* small_row, uint32_t swz) {
+  unsigned long long n2[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll 2
+  for (int c = 0; c < D / 8; ++c) {
+    const uint32_t off = (c >> 3) * kQBox + (static_cast<uint32_t>((c & 7) << 4) ^ swz);
+    const uint4 r = *reinterpret_cast<const uint4*>(raw_row + off), s = *reinterpret_cast<const uint4*>(small_row + off);
+    n2[0] = add_squares(n2[0], r.x | s.x);
+    n2[1] = add_squares(n2[1], r.y | s.y);
+    n2[2] = add_squares(n2[2], r.z | s.z);
+    n2[3] = add_squares(n2[3], r.w | s.w);
+  }
+  return (packed_total(n2[0]) + packed_total(n2[1])) + (packed_total(n2[2]) + packed_total(n2[3]));
+}
+
 // cnt[b] += the number of lanes whose mine == b (mine < 0: none), for every b < NB: five 6-bit counters per
 // warp sum, then one conflict-free addition per beacon (one atomic per lane would serialise).
 template <int NB>
@@ -312,7 +327,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
   __shared__ __align__(8) uint64_t sumready[kGroups], smallfree[kGroups], sumfull[kSums], cntready[kSums], sumfree[kSums];
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
-  __shared__ uint32_t seen_sh;               // largest |q|^2 below 2^(2 kMaxE) seen so far (fp32 bits)
+  __shared__ uint32_t seen_sh;               // largest element magnitude below 2^kMaxE seen so far (bf16 bits)
   // per instance in flight
   __shared__ uint32_t vmask_sh[kSlots];      // valid beacons (count > 0, nonzero centroid)
   __shared__ int exp_sh[kSlots];             // E; bit 8: a centroid norm is extreme, every query is re-decided
@@ -552,16 +567,14 @@ __global__ void __launch_bounds__(kUThreads, 1)
       ok = g < kGroups || mbar_wait(&smallfree[sb], ((g / kGroups) - 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
       if (!__all_sync(0xffffffffu, ok)) break;
 
-      // ---- the split of this query's elements, its squared norm and its extremes
+      // ---- the split of this query's elements and their extremes
       unsigned char* raw_row = stage_smem + st * C::kStageBytes + n * 128;
       uint32_t below = 0u;                 // bits of the elements below the operands' range
-      float qn2 = 0.f;
+      uint32_t qmax = 0u;                  // its largest element's magnitude (bf16 bits; NaN above all)
       if (n < rows) {
         const __nv_bfloat162 lim = as_bf162(pow2_bf16x2(E - kLargeBits));
         const __nv_bfloat162 lim_lo = as_bf162(pow2_bf16x2(E - kSmallBits));
-        __nv_bfloat162 n2[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) n2[k] = as_bf162(0u);
+        __nv_bfloat162 mx[2] = {as_bf162(0u), as_bf162(0u)};
         // four chunks are loaded before the first store: a chunk at a time would wait out its latencies
         // (rolled in between: the roles of this kernel compete for the instruction caches)
 #pragma unroll 1
@@ -581,21 +594,19 @@ __global__ void __launch_bounds__(kUThreads, 1)
             uint32_t s[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              const __nv_bfloat162 x2 = as_bf162(w[k]), a2 = __habs2(x2);
+              const __nv_bfloat162 a2 = __habs2(as_bf162(w[k]));
               s[k] = w[k] & __hlt2_mask(a2, lim);
               below |= w[k] & __hlt2_mask(a2, lim_lo);
-              n2[k] = __hfma2(x2, x2, n2[k]);
+              mx[k & 1] = __hmax2_nan(mx[k & 1], a2);
             }
             *reinterpret_cast<uint4*>(box_small + off[c]) = make_uint4(s[0], s[1], s[2], s[3]);
             st_shared_v4_if((s[0] | s[1]) | (s[2] | s[3]), box_raw + off[c], w[0] ^ s[0], w[1] ^ s[1], w[2] ^ s[2],
                             w[3] ^ s[3]);
           }
         }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float2 f = __bfloat1622float2(n2[k]);
-          qn2 += f.x + f.y;
-        }
+        const __nv_bfloat162 m2 = __hmax2_nan(mx[0], mx[1]);
+        const uint32_t mw = *reinterpret_cast<const uint32_t*>(&m2);
+        qmax = max(mw & 0xffffu, mw >> 16);
       } else {  // no query: nothing of a neighbour or of an earlier tile may enter the sums
         const uint4 z = make_uint4(0u, 0u, 0u, 0u);
         for (int c = 0; c < D / 8; ++c) {
@@ -604,19 +615,22 @@ __global__ void __launch_bounds__(kUThreads, 1)
           *reinterpret_cast<uint4*>(small_row + off) = z;
         }
       }
-      qn2 *= 1.1f;  // within a few percent (16 bf16 roundings per sum): taken too large
-      // |q| < 2^E bounds every element
-      const bool special = !(qn2 < __uint_as_float(static_cast<uint32_t>(2 * E + 127) << 23)) || (below & 0x7fff7fffu) != 0u;
+      const bool special = qmax >= (pow2_bf16x2(E) & 0xffffu) || (below & 0x7fff7fffu) != 0u;
       {
-        const uint32_t wmx =
-            __reduce_max_sync(0xffffffffu, qn2 < static_cast<float>(1 << (2 * kMaxE)) ? __float_as_uint(qn2) : 0u);
+        const uint32_t wmx = __reduce_max_sync(0xffffffffu, qmax < (pow2_bf16x2(kMaxE) & 0xffffu) ? qmax : 0u);
         if (lane == 0 && wmx > *reinterpret_cast<volatile uint32_t*>(&seen_sh)) atomicMax(&seen_sh, wmx);
       }
 
       // ---- decision
-      const bool wild = degenerate || !(qn2 > 1e-30f && qn2 < 1e30f);
-      const float margin = kScreenMargin * sqrt_approx(qn2);
-      const bool close = n < rows && vm != 0u && (wild || !(best - second > margin));
+      // |q| <= sqrt(d) max|q_i| rules most queries out; where it does not, |q| is formed in fp32
+      const float q_inf = __uint_as_float(qmax << 16);
+      const bool wild = degenerate || !(q_inf >= kTameLo && q_inf < kTameHi);
+      float margin = kScreenMargin * (D == 128 ? 11.313709f : 8.f) * q_inf;
+      bool close = n < rows && vm != 0u && (wild || !(best - second > margin));
+      if (__any_sync(0xffffffffu, close && !wild)) {
+        margin = kScreenMargin * sqrtf(row_norm2<D>(raw_row, small_row, swz));
+        close = close && (wild || !(best - second > margin));
+      }
       int my_b = n < rows ? bi : -1;
       uint32_t need = __ballot_sync(0xffffffffu, close);
       if (need) {  // rare: which beacons may be the exact best, while the dots are still there
@@ -849,9 +863,9 @@ __global__ void __launch_bounds__(kUThreads, 1)
           m = max(m, km_sh[w] & 0x7fffffffu);
           x |= km_sh[w] >> 31;
         }
-        // |q| < 2^E for what has been seen; before that four times the largest centroid
+        // every element seen is below 2^E; before that a guess from the largest centroid's norm
         const uint32_t seen = *reinterpret_cast<volatile uint32_t*>(&seen_sh);
-        int E = seen ? ((static_cast<int>(seen >> 23) - 127) >> 1) + 1 : ((static_cast<int>(m >> 23) - 127) >> 1) + 3;
+        int E = seen ? static_cast<int>(seen >> 7) - 126 : ((static_cast<int>(m >> 23) - 127) >> 1) + 2;
         E = E < kMinE ? kMinE : E > kMaxE ? kMaxE : E;
         vmask_sh[slot] = v;
         exp_sh[slot] = (E & 0xff) | (x ? 0x100 : 0);

@@ -45,6 +45,19 @@ __device__ __forceinline__ DF df_mul(DF a, DF b) {
 
 __device__ __forceinline__ bool df_gt(DF a, DF b) { return a.hi > b.hi || (a.hi == b.hi && a.lo > b.lo); }
 
+// Squared norm of a row of bf16 pairs in fp32: acc (two packed fp32 sums) plus the squares of the pair in
+// w (exact products, one rounding per addition), and the total of such a sum.
+__device__ __forceinline__ unsigned long long add_squares(unsigned long long acc, uint32_t w) {
+  const unsigned long long x =
+      static_cast<unsigned long long>(w << 16) | (static_cast<unsigned long long>(w & 0xffff0000u) << 32);
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(r) : "l"(x), "l"(acc));
+  return r;
+}
+__device__ __forceinline__ float packed_total(unsigned long long acc) {
+  return __uint_as_float(static_cast<uint32_t>(acc)) + __uint_as_float(static_cast<uint32_t>(acc >> 32));
+}
+
 // 1 / sqrt(a) for a double-float a > 0: the fp32 estimate y = rsqrtf(a.hi) (about 2^-22
 // relative) refined by one Newton-Raphson step for f(y) = 1 / y^2 - a,
 // y' = y + y (1 - a y^2) / 2, with the residual 1 - a y^2 formed in double-float
