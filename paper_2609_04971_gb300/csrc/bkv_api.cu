@@ -302,6 +302,7 @@ int bkv_create(const bkv_config* cfg, void* stream, bkv_ctx** out) {
   if ((e = cudaMemsetAsync(c->cent, 0, sizeof(float) * ni * s.nb * s.d + 0, c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->sums, 0, sizeof(double) * (c->cfps ? 1 : ni * s.nb * s.d), c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->spill, 0, sizeof(unsigned long long) * c->n_spill, c->stream)) != cudaSuccess ||
+      (e = cudaMemsetAsync(c->cbuf, 0, sizeof(__nv_bfloat16) * nh * c->b_max * s.d, c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->csize, 0, sizeof(int) * (nh ? nh : 1), c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->counts, 0, sizeof(long long) * ni * s.nb, c->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(c->err, 0, sizeof(int), c->stream)) != cudaSuccess) {
