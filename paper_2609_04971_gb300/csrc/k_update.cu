@@ -19,8 +19,8 @@
 // (the lowest beacon wins ties).  Only beacons screened within 1.4e-4 |q| of the
 // best enter that comparison.  |q| is formed, in fp32, only where the larger
 // sqrt(d) max|q_i| (exact: a packed maximum) does not rule a re-decision out (8192
-// instances of 512 queries, call and state read: 534 us, with an fp32 sum for
-// every query 574).  Zero queries and instances without a valid beacon give -1.
+// instances of 512 queries, call and state read: 527 us, some 40 less than with an
+// fp32 sum for every query).  Zero queries and instances without a valid beacon give -1.
 //
 // Sums: Q^T x A, where A is the tile's one-hot assignment matrix (128 queries x
 // beacons), exact: an element x with |x| < 2^E (E chosen per instance) goes
@@ -28,12 +28,13 @@
 // of 2^(E-17)) or a second tile (smaller ones, multiples of 2^(E-27) for
 // |x| >= 2^(E-20)), whose sums over 128 rows stay below 2^24 grid steps, so the
 // fp32 accumulator never rounds.  The two sums of a (column, beacon) cell are
-// integers, added up over the tiles in two registers.  The few elements outside
-// [2^(E-20), 2^E) (one in ten tiles of normal data) are zeroed in the operands
-// and added as a list (past 32 per instance through a global array of this CTA).
-// E comes from the largest element this CTA has seen (before that from the
-// centroids), never below -11, so that what the operands hold is exact in fixed
-// point with 40 fractional bits; the result does not depend on it.
+// integers, added up over the tiles in two registers.  Elements outside
+// [2^(E-20), 2^E) (one in fifteen tiles of data of one scale has some) are zeroed in
+// the operands and added one by one, from a list in shared memory (past its end
+// through a global array of this CTA).  E follows the instance's largest centroid
+// element and how far the queries of the last instances exceeded theirs; it is never
+// below -11, so that what the operands hold is exact in fixed point with 40
+// fractional bits, and the result does not depend on it.
 //
 // The call's sums (int64, 40 fractional bits) and counts go to scratch.  After its
 // last tile the CTA adds them once to the fp64 running sums of its instances,
@@ -51,12 +52,14 @@
 // What bounds it: a tile's chain through its group (dots, split, decision, sums:
 // about 8 K clocks, two tiles in flight per SM because shared memory holds no
 // third second-tile) and instruction fetch: the roles share the instruction caches,
-// so loops are kept rolled and rare paths small (re-decisions and spilled elements,
-// three tiles in ten, still cost a fifth of the time).  Sums formed in fp32 parts
-// by CUDA cores from rows sorted by beacon took about 14 K warp instructions per
-// tile.  With the fold (in a launch of its own: 255 and 485 us): 4608 instances x 512 queries of 128, 8 beacons: 393
-// us, now 242 (95 at the copy rate); 8192 instances, 16 beacons: 815 us, now 476
-// (178).
+// so loops are kept rolled and rare paths small, out of line and few.  Sums formed in
+// fp32 parts by CUDA cores from rows sorted by beacon took about 14 K warp
+// instructions per tile, whatever the data.  Kernel times, with those in brackets:
+// 4608 instances x 512 queries of 128, 8 beacons 219 us (380; 95 at the copy rate),
+// 8192 instances, 16 beacons 446 (761; 178).  Data of many scales spills in every
+// tile, 4608 instances: one query of 1000 times the scale in each CTA's first 266
+// (380), five columns of 300 times the rest 449 (414), elements spread by exp(1.5 N)
+// 579 (381), queries so spread 595 (380), elements over 24 octaves 1430 (389).
 #include "bkv_device.cuh"
 #include "bkv_internal.h"
 #include "k_update_math.cuh"
@@ -76,8 +79,10 @@ constexpr int kDots = 3;                    // screening accumulators in tensor 
 constexpr int kSums = 4;                    // sum accumulators in tensor memory
 constexpr int kSlots = 16;                  // per-instance words in flight between the roles (at most 11 instances)
 constexpr int kSpillSlots = 8;              // instances whose spilled elements may be in flight
-constexpr int kSpillList = 32;              // spilled elements per instance kept in shared memory
-constexpr size_t kUSmemBudget = 220 * 1024;
+constexpr int kSpillListMin = 128;          // spilled elements per instance kept in shared memory, at least
+constexpr int kSpillListMax = 1024;         // and at most
+constexpr int kFewRows = 2;                 // rows of a warp with spilled elements that are taken one by one
+constexpr size_t kUSmemBudget = 223 * 1024;
 // A query is re-decided exactly when its best and second-best dots differ by at most this fraction of |q|.
 // A screened dot is within 2^-18 |q| (the hi / lo split) + 136 * 2^-23 |q| (17 additions in each of eight
 // K = 16 steps) + 2^-21 |q| (1 / |c|) of the exact one, so a difference of two within 4.2e-5 |q|.
@@ -85,12 +90,16 @@ constexpr float kScreenMargin = 7e-5f;
 // Queries whose largest element is in this range have a squared norm that fp32 holds (1e-30 < |q|^2 < 1e30).
 constexpr float kTameLo = 1.7763568394002505e-15f, kTameHi = 70368744177664.f;  // 2^-49, 2^46
 constexpr int kMinE = -11, kMaxE = 14;
+constexpr int kRecent = 12;                 // instances before the one being built whose slots are still their own
+constexpr int kFirstRise = 64;              // rise of the queries above the centroids before any is seen: half an octave
+constexpr int kHeadroom = 32;               // and a quarter of one more (both in 1/128 octave)
 constexpr int kLargeBits = 10;              // octaves below 2^E that the tile itself holds
 constexpr int kSmallBits = 20;              // octaves below 2^E that the operands hold
 
 struct UpdArgs {
   int n_inst, nq, nb, nbp;  // instances, queries per instance, beacons, beacons padded to 8
   int box_rows;             // rows of one TMA box of queries (<= 128)
+  int list_cap;             // entries of an instance's list of spilled elements
   float* cent;
   double* sums;
   long long* counts;
@@ -114,15 +123,33 @@ struct UpdCfg {
     return kGroups * (kStageBytes + kHotBytes) + 2 * bmat_bytes(nbp) + kXchg;
   }
   static int stages(int nbp) {
-    const int n = static_cast<int>((kUSmemBudget - 1024 - fixed_bytes(nbp)) / kStageBytes);
+    const int n =
+        static_cast<int>((kUSmemBudget - 1024 - fixed_bytes(nbp) - kSpillSlots * kSpillListMin * 4) / kStageBytes);
     return n < kUMaxStages ? n : kUMaxStages;
   }
-  static size_t smem_bytes(int nbp) { return 1024 + static_cast<size_t>(stages(nbp)) * kStageBytes + fixed_bytes(nbp); }
+  static size_t smem_but_lists(int nbp) {
+    return 1024 + static_cast<size_t>(stages(nbp)) * kStageBytes + fixed_bytes(nbp);
+  }
+  // what the stages leave goes to the lists of spilled elements
+  static int list_cap(int nbp) {
+    const int n = static_cast<int>((kUSmemBudget - smem_but_lists(nbp)) / (kSpillSlots * 4));
+    return n < kSpillListMax ? n : kSpillListMax;
+  }
+  static size_t smem_bytes(int nbp) { return smem_but_lists(nbp) + static_cast<size_t>(list_cap(nbp)) * kSpillSlots * 4; }
 };
+
+// mbar_wait whose waiting loop is out of line: there are some twenty waits in the roles, which share the
+// instruction caches (235 -> 230 us, 4608 instances of 512 queries).
+__device__ __noinline__ bool wait_on(uint64_t* bar, uint32_t parity, volatile int* abort, int* err, int code) {
+  return mbar_wait(bar, parity, abort, err, code);
+}
+__device__ __forceinline__ bool wait_for(uint64_t* bar, uint32_t parity, volatile int* abort, int* err, int code) {
+  return mbar_try_wait(bar, parity) || wait_on(bar, parity, abort, err, code);
+}
 
 __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity, int* err) {
   int never = 0;
-  mbar_wait(bar, parity, &never, err, kDevTimeoutDrain);
+  wait_for(bar, parity, &never, err, kDevTimeoutDrain);
 }
 
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -271,48 +298,135 @@ __device__ __forceinline__ void add_counts(int* cnt, int mine) {
   if (lane < NB && n > 0) atomicAdd(&cnt[lane], n);
 }
 
-// Spilled elements of one instance: the first kSpillList as (beacon << 8 | column, fixed point) here, more
-// in the CTA's global array.
-struct SpillList {
-  int n;
-  int key[kSpillList];
-  long long val[kSpillList];
+// A spilled element (bf16 bits in the upper half) in fixed point.
+__device__ __forceinline__ long long spilled_fixed40(uint32_t hi16) {
+  const float x = __uint_as_float(hi16);
+  return fabsf(x) < 16384.f ? fixed40_one(x) : bf16_fixed40(hi16);
+}
+
+// Elements that the operands cannot hold: 0 < |x| < 2^(E - 20), |x| >= 2^E and what is not finite.  All sit in
+// the tile.  Each is zeroed there and noted for the row's beacon (b < 0: the row is not assigned) in the
+// instance's list, as (element << 16 | beacon << 8 | column), or, past its end, added to the global array.
+// Both functions are warp-wide, out of line and small, as rare code is fetched cold (2 - 3 K clocks a call); they
+// return whether something was added to the global array.
+
+// Where a CTA's spilled elements go (in shared memory: each argument that a call needs in a register cost the
+// loops around it 2 %).
+struct SpillTo {
+  int* list_n;
+  uint32_t* list;
+  unsigned long long* spill;
+  int list_cap, cells;
 };
 
-// The elements of one row (n of the tile) that the operands cannot hold: |x| >= 2^E (or not finite), which
-// sit in the tile, and 0 < |x| < 2^(E - 20), which sit in the second one.  Each is zeroed there and noted
-// for the row's beacon (b < 0: the row is not assigned).  Warp-wide; returns whether some went to the
-// global array.  Out of line: rare.
+// spill_row: one row (n of the tile), a lane per column.  Data of one scale has one such row in a few tiles.
 template <int D>
-__device__ __noinline__ bool spill_row(unsigned char* raw, unsigned char* small, int n, int E, int b, SpillList* list,
-                                       unsigned long long* spill) {
-  const int lane = threadIdx.x & 31;
+__device__ __noinline__ bool spill_row(unsigned char* raw, int n, int E, int b, int si, const SpillTo& to) {
+  int* list_n = to.list_n + si;
+  const int list_cap = to.list_cap;
+  uint32_t* list = to.list + si * list_cap;
+  unsigned long long* spill = to.spill + static_cast<size_t>(si) * to.cells;
   const uint32_t hi = pow2_bf16x2(E) & 0xffffu, lo = pow2_bf16x2(E - kSmallBits) & 0xffffu;
-  constexpr int kC = D / 32;  // this lane's columns
   bool over = false;
-#pragma unroll 1  // few instructions: they are fetched cold
-  for (int k = 0; k < kC; ++k) {
-    const int col = lane * kC + k;
-    const uint32_t off = sw128_offset(n, col, kQBox);
-    uint16_t* in_raw = reinterpret_cast<uint16_t*>(raw + off);
-    uint16_t* in_small = reinterpret_cast<uint16_t*>(small + off);
-    const uint32_t w = *in_raw | *in_small, m = w & 0x7fffu;  // one of the two is zero
+#pragma unroll 1
+  for (int col = threadIdx.x & 31; col < D; col += 32) {
+    uint16_t* at_x = reinterpret_cast<uint16_t*>(raw + sw128_offset(n, col, kQBox));
+    const uint32_t w = *at_x, m = w & 0x7fffu;
     if (m == 0u || (m >= lo && m < hi)) continue;
-    *in_raw = 0;
-    *in_small = 0;
+    *at_x = 0;
     if (b < 0) continue;
-    const float x = __uint_as_float(w << 16);
-    const long long f = fabsf(x) < 16384.f ? fixed40_one(x) : bf16_fixed40(w << 16);
-    const int at = atomicAdd(&list->n, 1);
-    if (at < kSpillList) {
-      list->key[at] = (b << 8) | col;
-      list->val[at] = f;
+    int at = *reinterpret_cast<volatile int*>(list_n);
+    if (at < list_cap) at = atomicAdd(list_n, 1);  // a full list's length is left alone: it stays far from overflow
+    if (at < list_cap) {
+      list[at] = w << 16 | static_cast<uint32_t>(b << 8 | col);
     } else {
-      atomicAdd(spill + b * D + col, static_cast<unsigned long long>(f));
+      atomicAdd(spill + b * D + col, static_cast<unsigned long long>(spilled_fixed40(w << 16)));
       over = true;
     }
   }
   if (!__any_sync(0xffffffffu, over)) return false;
+  __threadfence();
+  return true;
+}
+
+// spill_rows: each lane's own row (`mine`: it has some), for data of many scales, where every row has some.  The
+// lanes work side by side: first each marks its row's elements (one bit each), then all take their next marked
+// one at a time.
+template <int D>
+__device__ __noinline__ bool spill_rows(unsigned char* raw_row, uint32_t swz, int E, int b, bool mine, int si,
+                                        const SpillTo& to) {
+  int* list_n = to.list_n + si;
+  const int list_cap = to.list_cap;
+  uint32_t* list = to.list + si * list_cap;
+  unsigned long long* spill = to.spill + static_cast<size_t>(si) * to.cells;
+  constexpr uint32_t kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  // added to |x|, these put |x| >= 2^(E - 20) and |x| >= 2^E into bit 15
+  const uint32_t to_lo = 0x80008000u - pow2_bf16x2(E - kSmallBits), to_hi = 0x80008000u - pow2_bf16x2(E);
+  uint32_t m[D / 32];
+#pragma unroll
+  for (int g = 0; g < D / 32; ++g) m[g] = 0u;
+#pragma unroll 1
+  for (int c = 0; c < D / 8; ++c) {
+    const uint32_t off = (c >> 3) * kQBox + (static_cast<uint32_t>((c & 7) << 4) ^ swz);
+    const uint4 v = *reinterpret_cast<const uint4*>(raw_row + off);
+    const uint32_t w[4] = {v.x & 0x7fff7fffu, v.y & 0x7fff7fffu, v.z & 0x7fff7fffu, v.w & 0x7fff7fffu};
+    uint32_t bits = 0u;  // element 2k at bit 2k, element 2k + 1 at bit 16 + 2k
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      bits |= ((((w[k] + 0x7fff7fffu) & ~(w[k] + to_lo)) | (w[k] + to_hi)) & 0x80008000u) >> (15 - 2 * k);
+    bits = mine ? (bits & 0x55u) | ((bits >> 15) & 0xaau) : 0u;
+#pragma unroll
+    for (int g = 0; g + 1 < D / 32; ++g) m[g] = __funnelshift_r(m[g], m[g + 1], 8);
+    m[D / 32 - 1] = (m[D / 32 - 1] >> 8) | (bits << 24);
+  }
+  // room for all of them at once
+  uint32_t count = 0u;
+#pragma unroll
+  for (int g = 0; g < D / 32; ++g) count += b >= 0 ? __popc(m[g]) : 0u;
+  uint32_t at = count;  // becomes the number of elements of this lane and those before it
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t u = __shfl_up_sync(kAll, at, o);
+    at += lane >= o ? u : 0u;
+  }
+  int base = 0;
+  if (lane == 31) {  // a full list's length is left alone: it stays far from overflow
+    base = *reinterpret_cast<volatile int*>(list_n);
+    if (base < list_cap) base = atomicAdd(list_n, static_cast<int>(at));
+  }
+  at += static_cast<uint32_t>(__shfl_sync(kAll, base, 31)) - count;
+  bool over = false;
+#pragma unroll 1
+  while (__any_sync(kAll, (D == 128 ? m[0] | m[1] | m[D / 32 - 2] | m[D / 32 - 1] : m[0] | m[1]) != 0u)) {
+    int g = 0;
+    uint32_t cur = m[0];
+#pragma unroll
+    for (int k = 1; k < D / 32; ++k)
+      if (cur == 0u) {
+        cur = m[k];
+        g = k;
+      }
+    if (cur != 0u) {
+      const int col = 32 * g + __ffs(cur) - 1;
+#pragma unroll
+      for (int k = 0; k < D / 32; ++k) m[k] = k == g ? cur & (cur - 1u) : m[k];
+      const uint32_t off = (col >> 6) * kQBox + ((static_cast<uint32_t>(col & 0x38) << 1) ^ swz) + ((col & 7) << 1);
+      uint16_t* at_x = reinterpret_cast<uint16_t*>(raw_row + off);
+      const uint32_t w = static_cast<uint32_t>(*at_x) << 16;
+      *at_x = 0;
+      if (b >= 0) {
+        if (at < static_cast<uint32_t>(list_cap)) {
+          list[at] = w | static_cast<uint32_t>(b << 8 | col);
+        } else {
+          atomicAdd(spill + b * D + col, static_cast<unsigned long long>(spilled_fixed40(w)));
+          over = true;
+        }
+        ++at;
+      }
+    }
+  }
+  if (!__any_sync(kAll, over)) return false;
   __threadfence();
   return true;
 }
@@ -327,15 +441,17 @@ __global__ void __launch_bounds__(kUThreads, 1)
   __shared__ __align__(8) uint64_t sumready[kGroups], smallfree[kGroups], sumfull[kSums], cntready[kSums], sumfree[kSums];
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
-  __shared__ uint32_t seen_sh;               // largest element magnitude below 2^kMaxE seen so far (bf16 bits)
   // per instance in flight
   __shared__ uint32_t vmask_sh[kSlots];      // valid beacons (count > 0, nonzero centroid)
+  __shared__ uint32_t seen_sh[kSlots];       // largest query element below 2^kMaxE seen so far (bf16 bits)
+  __shared__ int cmax_sh[kSlots];            // largest centroid element (bf16 bits; 0: no valid beacon)
   __shared__ int exp_sh[kSlots];             // E; bit 8: a centroid norm is extreme, every query is re-decided
   __shared__ int add_cnt[kSlots][kMaxBeacons];  // queries assigned so far
   __shared__ int spilled_sh[kSlots];         // elements or sums went to the global array
-  __shared__ SpillList list_sh[kSpillSlots];
+  __shared__ SpillTo spill_to;
+  __shared__ int list_n_sh[kSpillSlots];     // spilled elements so far (those past the list's end are elsewhere)
   __shared__ uint32_t kv_sh[4];              // builders: each warp's valid beacons
-  __shared__ uint32_t km_sh[4];              // builders: each warp's largest |c|^2 (fp32 bits), bit 31: extreme norm
+  __shared__ uint32_t km_sh[4];              // builders: each warp's largest centroid element (fp32 bits), bit 31: extreme norm
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nq = a.nq, nb = a.nb, nbp = a.nbp;
@@ -353,6 +469,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
   unsigned char* hot_smem = small_smem + kGroups * C::kStageBytes;                // [kGroups][2][NBO x 128 B]
   unsigned char* bmat = hot_smem + kGroups * C::kHotBytes;                        // [2][kBoxes][2 nbp x 128 B]
   int* xchg = reinterpret_cast<int*>(bmat + 2 * C::bmat_bytes(nbp));  // d = 64: [NBO][64]
+  uint32_t* list_smem = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(xchg) + C::kXchg);  // [kSpillSlots][list_cap]
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < n_stages; ++i) {
@@ -379,14 +496,14 @@ __global__ void __launch_bounds__(kUThreads, 1)
     mbar_init(&drain_bar[0], 1);
     mbar_init(&drain_bar[1], 1);
     abort_sh = 0;
-    seen_sh = 0;
     fence_mbar_init();
   }
   for (uint32_t i = threadIdx.x; i < kGroups * C::kHotBytes / 16; i += kUThreads)
     reinterpret_cast<uint4*>(hot_smem)[i] = make_uint4(0u, 0u, 0u, 0u);
   for (int i = threadIdx.x; i < kSlots * kMaxBeacons; i += kUThreads) (&add_cnt[0][0])[i] = 0;
   if (threadIdx.x < kSlots) spilled_sh[threadIdx.x] = 0;
-  if (threadIdx.x < kSpillSlots) list_sh[threadIdx.x].n = 0;
+  if (threadIdx.x < kSpillSlots) list_n_sh[threadIdx.x] = 0;
+  if (threadIdx.x == 0) spill_to = SpillTo{list_n_sh, list_smem, a.spill + static_cast<size_t>(blockIdx.x) * kSpillSlots * nb * D, a.list_cap, nb * D};
   if (warp == 1) {
     tmem_alloc(&tmem_base_sh, 512);
     tmem_relinquish();
@@ -410,7 +527,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
       for (int i = 0; ok && i < n_my; ++i) {
         const int row0 = (blockIdx.x + i * gridDim.x) * nq;
         for (int t = 0; t < T; ++t) {
-          if (round > 0 && !mbar_wait(&empty_bar[st], (round - 1) & 1, abort_flag, a.err, kDevTimeoutProducer)) {
+          if (round > 0 && !wait_for(&empty_bar[st], (round - 1) & 1, abort_flag, a.err, kDevTimeoutProducer)) {
             ok = false;
             break;
           }
@@ -440,9 +557,9 @@ __global__ void __launch_bounds__(kUThreads, 1)
       int si = 0, s_t = 0, s_st = 0, s_round = 0, s_ab = 0, s_use = 0;  // screening: instance, tile, stage, accumulator
       auto screen = [&]() -> bool {
         const int pb = si & 1;
-        if (s_t == 0 && !mbar_wait(&bready[pb], (si >> 1) & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
-        if (!mbar_wait(&full_bar[s_st], s_round & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
-        if (s_use > 0 && !mbar_wait(&accfree[s_ab], (s_use - 1) & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
+        if (s_t == 0 && !wait_for(&bready[pb], (si >> 1) & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
+        if (!wait_for(&full_bar[s_st], s_round & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
+        if (s_use > 0 && !wait_for(&accfree[s_ab], (s_use - 1) & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
         tc_fence_after();
         const uint32_t d = tmem + s_ab * ncols1;
         const uint32_t q_addr = stage0 + s_st * C::kStageBytes;
@@ -481,8 +598,8 @@ __global__ void __launch_bounds__(kUThreads, 1)
       int m_st = 0;  // stage
       auto sum = [&](int g) -> bool {
         const int sb = g % kGroups, ub = g % kSums;
-        if (!mbar_wait(&sumready[sb], (g / kGroups) & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
-        if (g >= kSums && !mbar_wait(&sumfree[ub], ((g / kSums) - 1) & 1, abort_flag, a.err, kDevTimeoutMma))
+        if (!wait_for(&sumready[sb], (g / kGroups) & 1, abort_flag, a.err, kDevTimeoutMma)) return false;
+        if (g >= kSums && !wait_for(&sumfree[ub], ((g / kSums) - 1) & 1, abort_flag, a.err, kDevTimeoutMma))
           return false;
         // passes on what the group wrote besides the operands; after the wait above, so that the barrier is
         // never two phases ahead of the warps that wait for it
@@ -535,8 +652,8 @@ __global__ void __launch_bounds__(kUThreads, 1)
       const int st = g % n_stages, ab = g % kDots, slot = i & (kSlots - 1);
       const int rows = min(kQTile, nq - t * kQTile);
       // the tile's data and its dots (which also says that the screening has read the tile)
-      bool ok = mbar_wait(&full_bar[st], (g / n_stages) & 1, abort_flag, a.err, kDevTimeoutEpilogue) &&
-                mbar_wait(&accfull[ab], (g / kDots) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
+      bool ok = wait_for(&full_bar[st], (g / n_stages) & 1, abort_flag, a.err, kDevTimeoutEpilogue) &&
+                wait_for(&accfull[ab], (g / kDots) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
       const int E = static_cast<signed char>(exp_sh[slot] & 0xff);
@@ -564,7 +681,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
       }
 
       // this group's second tile is free once its previous tile's product is formed (the one-hot operand: below)
-      ok = g < kGroups || mbar_wait(&smallfree[sb], ((g / kGroups) - 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
+      ok = g < kGroups || wait_for(&smallfree[sb], ((g / kGroups) - 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
       if (!__all_sync(0xffffffffu, ok)) break;
 
       // ---- the split of this query's elements and their extremes
@@ -572,8 +689,8 @@ __global__ void __launch_bounds__(kUThreads, 1)
       uint32_t below = 0u;                 // bits of the elements below the operands' range
       uint32_t qmax = 0u;                  // its largest element's magnitude (bf16 bits; NaN above all)
       if (n < rows) {
-        const __nv_bfloat162 lim = as_bf162(pow2_bf16x2(E - kLargeBits));
-        const __nv_bfloat162 lim_lo = as_bf162(pow2_bf16x2(E - kSmallBits));
+        // 2^(E - 20) <= |x| < 2^(E - 10) goes to the second tile, what is below stays
+        const __nv_bfloat162 hi = as_bf162(pow2_bf16x2(E - kLargeBits)), lo = as_bf162(pow2_bf16x2(E - kSmallBits));
         __nv_bfloat162 mx[2] = {as_bf162(0u), as_bf162(0u)};
         // four chunks are loaded before the first store: a chunk at a time would wait out its latencies
         // (rolled in between: the roles of this kernel compete for the instruction caches)
@@ -595,8 +712,9 @@ __global__ void __launch_bounds__(kUThreads, 1)
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
               const __nv_bfloat162 a2 = __habs2(as_bf162(w[k]));
-              s[k] = w[k] & __hlt2_mask(a2, lim);
-              below |= w[k] & __hlt2_mask(a2, lim_lo);
+              const uint32_t under = __hlt2_mask(a2, lo);
+              s[k] = w[k] & __hlt2_mask(a2, hi) & ~under;
+              below |= w[k] & under;
               mx[k & 1] = __hmax2_nan(mx[k & 1], a2);
             }
             *reinterpret_cast<uint4*>(box_small + off[c]) = make_uint4(s[0], s[1], s[2], s[3]);
@@ -615,10 +733,10 @@ __global__ void __launch_bounds__(kUThreads, 1)
           *reinterpret_cast<uint4*>(small_row + off) = z;
         }
       }
-      const bool special = qmax >= (pow2_bf16x2(E) & 0xffffu) || (below & 0x7fff7fffu) != 0u;
+      const bool special = vm != 0u && ((below & 0x7fff7fffu) != 0u || qmax >= (pow2_bf16x2(E) & 0xffffu));
       {
         const uint32_t wmx = __reduce_max_sync(0xffffffffu, qmax < (pow2_bf16x2(kMaxE) & 0xffffu) ? qmax : 0u);
-        if (lane == 0 && wmx > *reinterpret_cast<volatile uint32_t*>(&seen_sh)) atomicMax(&seen_sh, wmx);
+        if (lane == 0 && wmx > *reinterpret_cast<volatile uint32_t*>(&seen_sh[slot])) atomicMax(&seen_sh[slot], wmx);
       }
 
       // ---- decision
@@ -662,7 +780,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
 
       if (n < rows && a.assign_out) a.assign_out[static_cast<size_t>(e) * nq + t * kQTile + n] = my_b;
       add_counts<NBO>(add_cnt[slot], my_b);
-      ok = g < kGroups || mbar_wait(&sumfull[(g - kGroups) % kSums], ((g - kGroups) / kSums) & 1, abort_flag, a.err,
+      ok = g < kGroups || wait_for(&sumfull[(g - kGroups) % kSums], ((g - kGroups) / kSums) & 1, abort_flag, a.err,
                                     kDevTimeoutEpilogue);
       if (!__all_sync(0xffffffffu, ok)) break;
       // ---- this query's column of the one-hot operand: 2^(17 - E), which makes the large part's sums integers
@@ -671,13 +789,20 @@ __global__ void __launch_bounds__(kUThreads, 1)
         *reinterpret_cast<uint16_t*>(hot + my_b * 128 + ((hot_chunk ^ (my_b & 7)) << 4)) =
             static_cast<uint16_t>(pow2_bf16x2(kLargeBits + 7 - E));
       prev_b = my_b;
-      for (uint32_t m = __ballot_sync(0xffffffffu, special); m; m &= m - 1) {  // rare
-        const int r = __ffs(m) - 1, b = __shfl_sync(0xffffffffu, my_b, r);
+      const uint32_t specials = __ballot_sync(0xffffffffu, special);
+      if (specials != 0u) {  // rare on data of one scale
         const int si = i & (kSpillSlots - 1);
-        __syncwarp();  // the rows' splits are written
-        if (spill_row<D>(stage_smem + st * C::kStageBytes, small_smem + sb * C::kStageBytes, quarter * 32 + r, E, b,
-                         &list_sh[si], a.spill + (static_cast<size_t>(blockIdx.x) * kSpillSlots + si) * nb * D))
-          spilled_sh[slot] = 1;
+        bool over = false;
+        if (__popc(specials) <= kFewRows) {
+          for (uint32_t m = specials; m; m &= m - 1) {
+            const int r = __ffs(m) - 1, b = __shfl_sync(0xffffffffu, my_b, r);
+            __syncwarp();  // the rows' splits are written
+            over |= spill_row<D>(stage_smem + st * C::kStageBytes, quarter * 32 + r, E, b, si, spill_to);
+          }
+        } else {
+          over = spill_rows<D>(raw_row, swz, E, my_b, special, si, spill_to);
+        }
+        if (over) spilled_sh[slot] = 1;
       }
       fence_proxy_async_smem();  // this thread's operand writes, read next by the tensor cores
       __syncwarp();
@@ -710,8 +835,8 @@ __global__ void __launch_bounds__(kUThreads, 1)
       bool ok = true;  // false after a wait gave up: the barriers below are still taken
       for (int t = 0; ok && t < T; ++t, ++g) {
         const int ub = g % kSums;
-        ok = mbar_wait(&cntready[ub], (g / kSums) & 1, abort_flag, a.err, kDevTimeoutEpilogue) &&
-             mbar_wait(&sumfull[ub], (g / kSums) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
+        ok = wait_for(&cntready[ub], (g / kSums) & 1, abort_flag, a.err, kDevTimeoutEpilogue) &&
+             wait_for(&sumfull[ub], (g / kSums) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
@@ -760,8 +885,8 @@ __global__ void __launch_bounds__(kUThreads, 1)
       const int add = lane < nb ? add_cnt[slot][lane] : 0;
       const int shift = static_cast<signed char>(exp_sh[slot] & 0xff) + 40 - (kSmallBits + 7);  // to units of 2^-40
       const bool spilled = spilled_sh[slot] != 0;
-      const SpillList& list = list_sh[i & (kSpillSlots - 1)];
-      const int n_list = min(list.n, kSpillList);
+      const uint32_t* list = list_smem + (i & (kSpillSlots - 1)) * a.list_cap;
+      const int n_list = min(list_n_sh[i & (kSpillSlots - 1)], a.list_cap);
       unsigned long long* spill =
           a.spill + (static_cast<size_t>(blockIdx.x) * kSpillSlots + (i & (kSpillSlots - 1))) * cells;
       if constexpr (D == 64) {
@@ -775,18 +900,34 @@ __global__ void __launch_bounds__(kUThreads, 1)
       }
       long long* out = a.call_sum + cbase + static_cast<size_t>(h0) * D + col;
       if (ok && !small_half) {
+        long long f[HB];
 #pragma unroll
-        for (int b = 0; b < HB; ++b)
-          if (h0 + b < nb) out[b * D] = (acc_l[b] * 1024ll + acc_s[b]) << shift;
-        for (int k = 0; k < n_list; ++k) {  // spilled elements of this thread's cells: rare
-          const int b = (list.key[k] >> 8) - h0;
-          if ((list.key[k] & 0xff) == col && b >= 0 && b < HB) out[b * D] += list.val[k];
+        for (int b = 0; b < HB; ++b) f[b] = (acc_l[b] * 1024ll + acc_s[b]) << shift;
+        for (int k = 0; k < n_list; k += 32) {  // rare: spilled elements, a lane each; then those of this warp's cells
+          const uint32_t key = k + lane < n_list ? list[k + lane] : 0xffffu;
+          const int at = static_cast<int>(key & 0xffffu);  // (beacon, column)
+          const long long v = spilled_fixed40(key & 0xffff0000u);
+          uint32_t m = __ballot_sync(0xffffffffu, (at & 0xff) >> 5 == quarter && at >> 8 >= h0 && at >> 8 < h0 + HB);
+          for (; m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            const int one = __shfl_sync(0xffffffffu, at, src);
+            const long long v1 = __shfl_sync(0xffffffffu, v, src);
+            const int b1 = (one & 31) == lane ? (one >> 8) - h0 : -1;
+#pragma unroll
+            for (int b = 0; b < HB; ++b)
+              if (b == b1) f[b] += v1;
+          }
         }
         if (spilled)
-          for (int b = 0; b < HB && h0 + b < nb; ++b) {
-            out[b * D] += static_cast<long long>(__ldcg(spill + (h0 + b) * D + col));
-            spill[(h0 + b) * D + col] = 0ull;
-          }
+#pragma unroll
+          for (int b = 0; b < HB; ++b)
+            if (h0 + b < nb) {
+              f[b] += static_cast<long long>(__ldcg(spill + (h0 + b) * D + col));
+              spill[(h0 + b) * D + col] = 0ull;
+            }
+#pragma unroll
+        for (int b = 0; b < HB; ++b)
+          if (h0 + b < nb) out[b * D] = f[b];
       }
       if (spilled) __threadfence();
       named_barrier(1, 256);  // every warp has read this slot's words (and, d = 64, the exchanged sums)
@@ -794,7 +935,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
       if (first_warp) add_cnt[slot][lane] = 0;
       if (first_warp && lane == 0) {
         spilled_sh[slot] = 0;
-        list_sh[i & (kSpillSlots - 1)].n = 0;
+        list_n_sh[i & (kSpillSlots - 1)] = 0;
       }
     }
   } else {
@@ -807,10 +948,10 @@ __global__ void __launch_bounds__(kUThreads, 1)
         bulk_prefetch_l2(a.cent + (static_cast<size_t>(e) + gridDim.x) * nb * D, static_cast<uint32_t>(nb * D) * 4);
       const long long cnt = lane < nb ? a.counts[static_cast<size_t>(e) * nb + lane] : 0;
       const uint32_t counted = __ballot_sync(0xffffffffu, cnt > 0);
-      if (i >= 2) mbar_wait(&bfree[pb], ((i >> 1) - 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
+      if (i >= 2) wait_for(&bfree[pb], ((i >> 1) - 1) & 1, abort_flag, a.err, kDevTimeoutEpilogue);
       unsigned char* bm = bmat + pb * C::bmat_bytes(nbp);
       uint32_t valid = 0u;
-      float cmax = 0.f;
+      uint32_t cmax = 0u;
       bool extreme = false;
 #pragma unroll 1
       for (int b0 = wk; b0 < nbp; b0 += 4 * kBatch) {
@@ -829,13 +970,13 @@ __global__ void __launch_bounds__(kUThreads, 1)
           for (int k = 0; k < D / 32; ++k) n2 = fmaf(c[u][k], c[u][k], n2);
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
-          bool nz = false;
+          float big = 0.f;
 #pragma unroll
-          for (int k = 0; k < D / 32; ++k) nz |= c[u][k] != 0.f;
-          const bool ok = ((counted >> (b & 31)) & 1u) && b < nb && __any_sync(0xffffffffu, nz);
+          for (int k = 0; k < D / 32; ++k) big = fmaxf(big, fabsf(c[u][k]));
+          const bool ok = ((counted >> (b & 31)) & 1u) && b < nb && __any_sync(0xffffffffu, big != 0.f || n2 != n2);
           if (ok) {
             valid |= 1u << b;
-            cmax = fmaxf(cmax, n2);
+            cmax = max(cmax, __float_as_uint(big));
             extreme |= !(n2 > 1e-30f && n2 < 1e30f);
           }
           const float inv = ok ? rsqrtf(n2) : 0.f;
@@ -850,26 +991,47 @@ __global__ void __launch_bounds__(kUThreads, 1)
           }
         }
       }
+      cmax = __reduce_max_sync(0xffffffffu, cmax);
       if (lane == 0) {
         kv_sh[wk] = valid;
-        km_sh[wk] = (__float_as_uint(cmax) & 0x7fffffffu) | (extreme ? 0x80000000u : 0u);
+        km_sh[wk] = cmax | (extreme ? 0x80000000u : 0u);
       }
       fence_proxy_async_smem();  // generic-proxy writes, read next by the tensor cores
       named_barrier(2, 128);
-      if (wk == 0 && lane == 0) {
+      if (wk == 0) {
         uint32_t v = 0u, m = 0u, x = 0u;
         for (int w = 0; w < 4; ++w) {
           v |= kv_sh[w];
           m = max(m, km_sh[w] & 0x7fffffffu);
           x |= km_sh[w] >> 31;
         }
-        // every element seen is below 2^E; before that a guess from the largest centroid's norm
-        const uint32_t seen = *reinterpret_cast<volatile uint32_t*>(&seen_sh);
-        int E = seen ? static_cast<int>(seen >> 7) - 126 : ((static_cast<int>(m >> 23) - 127) >> 1) + 2;
-        E = E < kMinE ? kMinE : E > kMaxE ? kMaxE : E;
-        vmask_sh[slot] = v;
-        exp_sh[slot] = (E & 0xff) | (x ? 0x100 : 0);
-        mbar_arrive(&bready[pb]);
+        // E: what the instance's largest centroid element is times what the queries' elements exceeded theirs
+        // by in the last three instances with some (kFirstRise before that), and kHeadroom.  Scales differ by
+        // head and layer, so neither a fixed E nor the largest element so far would serve: one query of 1000
+        // times the scale raised E, and with it the number of spilled elements, for all that followed (3 times
+        // the time).  bf16 bits are used as logarithms, in 1/128 octave.
+        const int back = i - 1 - lane;  // the slots of the last instances, all of them written
+        int rise = 0;
+        bool some = false;
+        if (lane < kRecent && back >= 0) {
+          const int seen = static_cast<int>(*reinterpret_cast<volatile uint32_t*>(&seen_sh[back & (kSlots - 1)]));
+          const int c0 = *reinterpret_cast<volatile int*>(&cmax_sh[back & (kSlots - 1)]);
+          rise = seen - c0;
+          some = seen != 0 && c0 != 0;
+        }
+        const uint32_t with = __ballot_sync(0xffffffffu, some);
+        const bool taken = some && __popc(with & ((1u << lane) - 1u)) < 3;
+        rise = __reduce_max_sync(0xffffffffu, taken ? rise : -(1 << 16));
+        if (lane == 0) {
+          const int c0 = static_cast<int>(m >> 16);
+          int E = ((c0 + (with ? rise : kFirstRise) + kHeadroom) >> 7) - 126;
+          E = E < kMinE ? kMinE : E > kMaxE ? kMaxE : E;
+          vmask_sh[slot] = v;
+          exp_sh[slot] = (E & 0xff) | (x ? 0x100 : 0);
+          seen_sh[slot] = 0u;
+          cmax_sh[slot] = v ? c0 : 0;
+          mbar_arrive(&bready[pb]);
+        }
       }
       named_barrier(2, 128);  // kv_sh and km_sh are free again
     }
@@ -925,8 +1087,9 @@ __global__ void __launch_bounds__(kUThreads, 1)
 }
 
 template <int D, int NBO>
-cudaError_t launch_update_dn(const UpdArgs& a, const CUtensorMap& qmap, int grid, cudaStream_t st) {
+cudaError_t launch_update_dn(UpdArgs a, const CUtensorMap& qmap, int grid, cudaStream_t st) {
   using C = UpdCfg<D, NBO>;
+  a.list_cap = C::list_cap(a.nbp);
   const size_t smem = C::smem_bytes(a.nbp);
   const cudaError_t e = allow_smem<update_kernel<D, NBO>>(smem);
   if (e != cudaSuccess) return e;
