@@ -24,13 +24,19 @@
 //     (1 / |q_j|) (1 / |q_r|).  Rows are compared as the doubles those
 //     double-floats equal, so every pick equals that of the fp64 definition
 //     except at ties below ~1e-13 relative (lowest index on exact ties).  A
-//     row's exact S is kept with the number of picks it covers, so that many
-//     tied rows cost no more than an all-exact run.  A row whose squared norm is
-//     far from 1 (or not finite) sends every decision of its instance there.
+//     row's exact S is kept with the number of picks it covers.  Of rows with
+//     the same bits (repeated tokens, zero rows) only the first is compared.
+//     Where more than half of the rows left are compared exactly, as with rows
+//     all closer than the screening can tell apart, nothing is screened any
+//     more; nor is it in an instance with a row whose squared norm is far from 1
+//     (or not finite).
 //
 // What bounds it: issue slots and the two barriers per pick; the rows cross HBM
-// once.  All decisions in double-float arithmetic took 1212 us for 4608
-// instances of 256 rows of 128 (8 picks); screened it takes 210 us (its rows cross HBM in 45).
+// once.  Kernel and state read, 4608 instances of 256 rows of 128, 8 picks, with
+// all decisions in double-float arithmetic in brackets: 214 us (1217; the rows
+// cross HBM in 45); all rows equal 416 (1216), each four times 311 (1218), three in
+// four zero 502 (483), all within 0.01 of one direction 1103 (1215), one row of
+// extreme norm 1017 (1217).
 #include "bkv_device.cuh"
 #include "bkv_internal.h"
 #include "k_update_math.cuh"
@@ -41,6 +47,7 @@ namespace {
 constexpr size_t kFpsResident = 200 * 1024;  // rows stay in shared memory up to this many bytes
 constexpr float kCosEps = 3.0517578125e-05f;  // 2^-15: bound on the error of a screened cosine
 constexpr uint32_t kFpsFull = 0xffffffffu;
+constexpr int kCovers = 0x3f, kPicked = 0x40, kHasInv = 0x80;  // per-row bits (at most 31 picks are covered)
 
 __device__ __forceinline__ double bf(const __nv_bfloat16 v) { return static_cast<double>(__bfloat162float(v)); }
 
@@ -86,28 +93,6 @@ __device__ void block_argmin(double v, int i, double* red_v, int* red_i, double&
   __syncthreads();
 }
 
-// Sum over this row's elements of x_k * y_k for bf16 rows (two 16-byte loads per 8
-// elements): each product of two bf16 values is exact in fp32, and the products are
-// summed in double-float arithmetic in two interleaved chains (even and odd groups of 8).
-template <int D>
-__device__ __forceinline__ DF dot_bf16(const __nv_bfloat16* x, const __nv_bfloat16* y) {
-  DF a0{0.f, 0.f}, a1{0.f, 0.f};
-#pragma unroll 2
-  for (int k = 0; k < D; k += 16) {
-    const uint4 xa = *reinterpret_cast<const uint4*>(x + k), xb = *reinterpret_cast<const uint4*>(x + k + 8);
-    const uint4 ya = *reinterpret_cast<const uint4*>(y + k), yb = *reinterpret_cast<const uint4*>(y + k + 8);
-    const uint32_t wx[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
-    const uint32_t wy[8] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      DF& acc = i < 4 ? a0 : a1;
-      acc = df_add(acc, DF{__fmul_rn(__uint_as_float(wx[i] << 16), __uint_as_float(wy[i] << 16)), 0.f});
-      acc = df_add(acc, DF{__fmul_rn(__uint_as_float(wx[i] & 0xffff0000u), __uint_as_float(wy[i] & 0xffff0000u)), 0.f});
-    }
-  }
-  return df_add(a0, a1);
-}
-
 // A double-float as the double it equals (hi + lo needs at most 48 significant bits).
 __device__ __forceinline__ double df_to_double(DF v) {
   return __dadd_rn(static_cast<double>(v.hi), static_cast<double>(v.lo));
@@ -133,7 +118,7 @@ __host__ __device__ inline FpsLayout fps_layout(int N, int D, int threads, bool 
   o += 4 * np;
   l.list = o;  // uint16 [np]: rows to compare exactly
   o += 2 * np;
-  l.kx = o;  // uint8 [np]: picks that sx covers; bit 7: inv is set
+  l.kx = o;  // uint8 [np]: picks that sx covers (kCovers); kPicked; kHasInv: inv is set
   o += np;
   l.total = o;
   return l;
@@ -162,6 +147,20 @@ __device__ __forceinline__ float sum2(unsigned long long v) {
   return __uint_as_float(static_cast<uint32_t>(v)) + __uint_as_float(static_cast<uint32_t>(v >> 32));
 }
 
+// Element k of row j.
+template <int D, bool RES>
+__device__ __forceinline__ float element(const uint32_t* xs, const __nv_bfloat16* x, int j, int k) {
+  const uint32_t w = row_word<D, RES>(xs, x, j, k >> 1);
+  return __uint_as_float((k & 1) ? w & 0xffff0000u : w << 16);
+}
+
+// The first row that is not picked.
+__device__ __forceinline__ int first_left(const unsigned char* kx, int N) {
+  for (int j = 0; j < N; ++j)
+    if (!(kx[j] & kPicked)) return j;
+  return 0;
+}
+
 // 16-byte chunk c of row j.
 template <int D, bool RES>
 __device__ __forceinline__ uint4 row_chunk(const uint32_t* xs, const __nv_bfloat16* x, int j, int c) {
@@ -171,6 +170,38 @@ __device__ __forceinline__ uint4 row_chunk(const uint32_t* xs, const __nv_bfloat
   } else {
     return reinterpret_cast<const uint4*>(x)[static_cast<size_t>(j) * (D / 8) + c];
   }
+}
+
+// Sum of x_k * y_k over the elements of rows i and j: each product of two bf16 values is exact in fp32, and the
+// products are summed in double-float arithmetic in two interleaved chains (even and odd chunks of 8).
+template <int D, bool RES>
+__device__ __forceinline__ DF row_dot(const uint32_t* xs, const __nv_bfloat16* x, int i, int j) {
+  DF a0{0.f, 0.f}, a1{0.f, 0.f};
+#pragma unroll 2
+  for (int c = 0; c < D / 8; c += 2) {
+    const uint4 xa = row_chunk<D, RES>(xs, x, i, c), xb = row_chunk<D, RES>(xs, x, i, c + 1);
+    const uint4 ya = row_chunk<D, RES>(xs, x, j, c), yb = row_chunk<D, RES>(xs, x, j, c + 1);
+    const uint32_t wx[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+    const uint32_t wy[8] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      DF& acc = k < 4 ? a0 : a1;
+      acc = df_add(acc, DF{__fmul_rn(__uint_as_float(wx[k] << 16), __uint_as_float(wy[k] << 16)), 0.f});
+      acc = df_add(acc, DF{__fmul_rn(__uint_as_float(wx[k] & 0xffff0000u), __uint_as_float(wy[k] & 0xffff0000u)), 0.f});
+    }
+  }
+  return df_add(a0, a1);
+}
+
+// Whether rows i and j hold the same bits.
+template <int D, bool RES>
+__device__ __forceinline__ bool same_row(const uint32_t* xs, const __nv_bfloat16* x, int i, int j) {
+#pragma unroll 1
+  for (int c = 0; c < D / 8; ++c) {
+    const uint4 a = row_chunk<D, RES>(xs, x, i, c), b = row_chunk<D, RES>(xs, x, j, c);
+    if (((a.x ^ b.x) | (a.y ^ b.y) | (a.z ^ b.z) | (a.w ^ b.w)) != 0u) return false;
+  }
+  return true;
 }
 
 // Products of the 16 rows r0 .. r0 + 15 (rows of N and more are zero) with the 8 columns whose
@@ -243,7 +274,7 @@ __device__ __forceinline__ float first_eps(int N, int chain, float u_norm) {
 // NW warps, MT 16-row tiles per warp (warp w takes tiles w, w + NW, ...).  Lane 4 g of a warp owns the
 // rows g and g + 8 of each of its tiles: their screening values stay in its registers.
 template <int D, int NW, int MT, bool RES>
-__global__ void __launch_bounds__(32 * NW, MT == 2 ? 24 / NW : MT == 4 ? 3 : 1)
+__global__ void __launch_bounds__(32 * NW, MT == 2 ? 24 / NW : MT == 4 ? (NW == 4 ? 3 : 2) : 1)
     fps_init_kernel(const __nv_bfloat16* __restrict__ q, int N, int nb, float* __restrict__ cent,
                     double* __restrict__ sums, long long* __restrict__ counts) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -256,7 +287,7 @@ __global__ void __launch_bounds__(32 * NW, MT == 2 ? 24 / NW : MT == 4 ? 3 : 1)
   __shared__ int picks[kMaxBeacons];
   __shared__ float u2_sh[NW];          // squared norm of the sum, per warp
   __shared__ uint32_t min_sh[2];       // order key of the smallest screening value, by pick parity
-  __shared__ int cnt_sh[2], wild_sh, n_pinv_sh;
+  __shared__ int cnt_sh[2], wild_sh, n_pinv_sh, low_sh, left_sh;
 
   constexpr int T = 32 * NW;
   const int e = blockIdx.x, tid = threadIdx.x;
@@ -447,26 +478,57 @@ __global__ void __launch_bounds__(32 * NW, MT == 2 ? 24 / NW : MT == 4 ? 3 : 1)
     __syncthreads();
     return cnt_sh[k & 1];
   };
+  // Drops from the n listed rows those with the same bits as a listed row of a lower index: they tie with it
+  // exactly and lose.  Two such rows are looked for (repeated tokens, zero rows); returns what is left.
+  auto drop_repeats = [&](int n) -> int {
+    int above = -1;
+#pragma unroll 1
+    for (int round = 0; round < 2 && n > 1; ++round) {
+      if (tid == 0) {
+        low_sh = 0x7fffffff;
+        left_sh = 0;
+      }
+      __syncthreads();
+      int low = 0x7fffffff;
+      for (int c = tid; c < n; c += T) low = list[c] > above ? min(low, static_cast<int>(list[c])) : low;
+      low = __reduce_min_sync(kFpsFull, low);
+      if (lane == 0) atomicMin(&low_sh, low);
+      __syncthreads();
+      low = low_sh;
+      if (low == 0x7fffffff) break;  // block-uniform
+      for (int c0 = 0; c0 < n; c0 += T) {
+        const int j = c0 + tid < n ? list[c0 + tid] : -1;
+        const bool stays = j >= 0 && (j <= low || !same_row<D, RES>(xs, x, j, low));
+        __syncthreads();  // this part of the list is read: what stays of it moves to the front
+        if (stays) list[atomicAdd(&left_sh, 1)] = static_cast<uint16_t>(j);
+      }
+      __syncthreads();
+      n = left_sh;
+      above = low;
+      __syncthreads();
+    }
+    return n;
+  };
   float u2 = u2_sh[0];
 #pragma unroll
   for (int w = 1; w < (D / 2 + 31) / 32; ++w) u2 += u2_sh[w];
-  int n_cand = collect(2.f * first_eps<D>(N, chain, sqrtf(u2)), 0);
+  int n_cand = drop_repeats(collect(2.f * first_eps<D>(N, chain, sqrtf(u2)), 0));
+  bool dense = wild;  // every row not picked yet is compared exactly, nothing is screened
   int r;
   if (n_cand == 1) {
     r = list[0];
   } else {
     // exact: 1 / |q_j| of every row, u = sum_j q_j / |q_j|, then the candidates
     for (int j = tid; j < N; j += T) {
-      const DF n2 = dot_bf16<D>(x + static_cast<size_t>(j) * D, x + static_cast<size_t>(j) * D);
+      const DF n2 = row_dot<D, RES>(xs, x, j, j);
       bool plain = true;
       inv[j] = n2.hi > 0.f ? centroid_inv_norm(n2, n2.hi, plain) : DF{0.f, 0.f};
-      kx[j] = 0x80;
+      kx[j] = kHasInv;
     }
     __syncthreads();
     for (int k = tid; k < D; k += T) {
       DF a{0.f, 0.f};
-      for (int j = 0; j < N; ++j)
-        a = df_add(a, df_mul(DF{__bfloat162float(x[static_cast<size_t>(j) * D + k]), 0.f}, inv[j]));
+      for (int j = 0; j < N; ++j) a = df_add(a, df_mul(DF{element<D, RES>(xs, x, j, k), 0.f}, inv[j]));
       u[k] = a;
     }
     __syncthreads();
@@ -477,8 +539,7 @@ __global__ void __launch_bounds__(32 * NW, MT == 2 ? 24 / NW : MT == 4 ? 3 : 1)
       DF t{0.f, 0.f};
       if (inv[i].hi > 0.f) {
         DF a{0.f, 0.f};
-        for (int k = 0; k < D; ++k)
-          a = df_add(a, df_mul(DF{__bfloat162float(x[static_cast<size_t>(i) * D + k]), 0.f}, u[k]));
+        for (int k = 0; k < D; ++k) a = df_add(a, df_mul(DF{element<D, RES>(xs, x, i, k), 0.f}, u[k]));
         t = df_mul(a, inv[i]);
       }
       const double tv = df_to_double(t);
@@ -491,116 +552,128 @@ __global__ void __launch_bounds__(32 * NW, MT == 2 ? 24 / NW : MT == 4 ? 3 : 1)
     block_argmin(best_v, best_i, red_v, red_i, pv, r);
     if (r >= N) r = n_cand > 0 ? list[0] : 0;  // no finite value at all
   }
-  if (tid == 0) picks[0] = r;
+  if (tid == 0) {
+    picks[0] = r;
+    kx[r] |= kPicked;
+  }
 
   // ---- S_j = max over the picks of cos(q_j, q_pick), one pick at a time
   const uint32_t zero_chunk = smem_u32(zero_sh);
   for (int k = 1; k < nb; ++k) {
-    const float inv_r = inv32[r];
-    pick_fragments<D, RES>(xs, x, r, zero_chunk, bfrag);
-    if (k == 1) {
+    if (!dense) {
+      const float inv_r = inv32[r];
+      pick_fragments<D, RES>(xs, x, r, zero_chunk, bfrag);
+      if (k == 1) {
 #pragma unroll
-      for (int m = 0; m < MT; ++m)
+        for (int m = 0; m < MT; ++m)
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
-          S[m][h] = (lane & 3) == 0 && row0 + 16 * m * NW + 8 * h < N ? -INFINITY : INFINITY;
-    }
-    if (((r >> 4) & (NW - 1)) == warp) {  // r is one of this warp's rows
-#pragma unroll
-      for (int m = 0; m < MT; ++m)
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-          if (row0 + 16 * m * NW + 8 * h == r && (lane & 3) == 0) {
-            S[m][h] = INFINITY;
-            iv[m][h] = 0.f;
-          }
-    }
-    wmin = INFINITY;
-#pragma unroll
-    for (int m = 0; m < MT; ++m) {
-      const int r0 = 16 * (warp + m * NW);
-      if (r0 >= np) continue;  // warp-uniform
-      float d[4];
-      tile_products<D, RES>(xs, x, N, r0, taddr, m * kTileStep, bfrag, d);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        S[m][h] = fmaxf(S[m][h], d[2 * h] * inv_r * iv[m][h]);
-        wmin = fminf(wmin, S[m][h]);
+          for (int h = 0; h < 2; ++h)
+            S[m][h] = (lane & 3) == 0 && row0 + 16 * m * NW + 8 * h < N ? -INFINITY : INFINITY;
       }
+      if (((r >> 4) & (NW - 1)) == warp) {  // r is one of this warp's rows
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (row0 + 16 * m * NW + 8 * h == r && (lane & 3) == 0) {
+              S[m][h] = INFINITY;
+              iv[m][h] = 0.f;
+            }
+      }
+      wmin = INFINITY;
+#pragma unroll
+      for (int m = 0; m < MT; ++m) {
+        const int r0 = 16 * (warp + m * NW);
+        if (r0 >= np) continue;  // warp-uniform
+        float d[4];
+        tile_products<D, RES>(xs, x, N, r0, taddr, m * kTileStep, bfrag, d);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          S[m][h] = fmaxf(S[m][h], d[2 * h] * inv_r * iv[m][h]);
+          wmin = fminf(wmin, S[m][h]);
+        }
+      }
+      n_cand = collect(2.f * kCosEps, k);
+      if (n_cand > 1) n_cand = drop_repeats(n_cand);
+    } else {
+      __syncthreads();  // the last pick is marked
+      n_cand = N - k;
     }
-    n_cand = collect(2.f * kCosEps, k);
-    if (n_cand == 1) {
+    if (n_cand == 1 && !dense) {
       r = list[0];
     } else {
       // exact 1 / |q| of the picks so far, then each candidate's S over the picks it does not cover yet
-      for (int m = n_pinv_sh + tid; m < k; m += T) {
-        const __nv_bfloat16* xp = x + static_cast<size_t>(picks[m]) * D;
-        const DF n2 = dot_bf16<D>(xp, xp);
-        bool plain = true;
-        pinv[m] = n2.hi > 0.f ? centroid_inv_norm(n2, n2.hi, plain) : DF{0.f, 0.f};
-      }
-      __syncthreads();
-      if (tid == 0) n_pinv_sh = k;
       auto inv_of = [&](int j) -> DF {
-        if (kx[j] & 0x80) return inv[j];
-        const __nv_bfloat16* xj = x + static_cast<size_t>(j) * D;
-        const DF n2 = dot_bf16<D>(xj, xj);
+        if (kx[j] & kHasInv) return inv[j];
+        const DF n2 = row_dot<D, RES>(xs, x, j, j);
         bool plain = true;
         return n2.hi > 0.f ? centroid_inv_norm(n2, n2.hi, plain) : DF{0.f, 0.f};
       };
+      for (int m = n_pinv_sh + tid; m < k; m += T) pinv[m] = inv_of(picks[m]);
+      __syncthreads();
+      if (tid == 0) n_pinv_sh = k;
       auto cosine = [&](int j, DF inv_j, int m) -> double {
         if (!(inv_j.hi > 0.f && pinv[m].hi > 0.f)) return 0.0;
-        return df_to_double(
-            df_mul(df_mul(dot_bf16<D>(x + static_cast<size_t>(j) * D, x + static_cast<size_t>(picks[m]) * D), inv_j),
-                   pinv[m]));
+        return df_to_double(df_mul(df_mul(row_dot<D, RES>(xs, x, j, picks[m]), inv_j), pinv[m]));
       };
-      if (n_cand <= 4 * NW) {  // a few: a warp per candidate, a lane per pick
+      double v = INFINITY;
+      int vi = 0x7fffffff;
+      if (!dense && n_cand <= 4 * NW) {  // a few: a warp per candidate, a lane per pick
         for (int c = warp; c < n_cand; c += NW) {
           const int j = list[c];
-          const int k0 = kx[j] & 0x7f;
+          const int k0 = kx[j] & kCovers;
           const DF inv_j = inv_of(j);
           const double cv = lane >= k0 && lane < k ? cosine(j, inv_j, lane) : 0.0;
-          double S = k0 ? Sx[j] : 0.0;
+          double Sj = k0 ? Sx[j] : 0.0;
           for (int m = k0; m < k; ++m) {
             const double cm = __shfl_sync(kFpsFull, cv, m);
-            if (m == 0 || cm > S) S = cm;
+            if (m == 0 || cm > Sj) Sj = cm;
           }
           __syncwarp();
           if (lane == 0) {
-            Sx[j] = S;
+            Sx[j] = Sj;
             inv[j] = inv_j;
-            kx[j] = static_cast<unsigned char>(0x80 | k);
+            kx[j] = static_cast<unsigned char>(kHasInv | k);
+          }
+          if (Sj < v || (Sj == v && j < vi)) {
+            v = Sj;
+            vi = j;
           }
         }
-      } else {  // many (tied rows): a thread per candidate
-        for (int c = tid; c < n_cand; c += T) {
-          const int j = list[c];
-          const DF inv_j = inv_of(j);
-          double S = Sx[j];
-          for (int m = kx[j] & 0x7f; m < k; ++m) {
-            const double cm = cosine(j, inv_j, m);
-            if (m == 0 || cm > S) S = cm;
+      } else {  // many: a thread per candidate
+        for (int c = tid; c < (dense ? N : n_cand); c += T) {
+          const int j = dense ? c : list[c];
+          if (dense && (kx[j] & kPicked)) continue;
+          bool has_inv = (kx[j] & kHasInv) != 0;
+          DF inv_j = inv[j];
+          double Sj = Sx[j];
+          for (int m = kx[j] & kCovers; m < k; ++m) {
+            if (!has_inv && pinv[m].hi > 0.f) {  // 0 with a zero pick: no norm is needed
+              inv_j = inv_of(j);
+              has_inv = true;
+            }
+            const double cm = has_inv ? cosine(j, inv_j, m) : 0.0;
+            if (m == 0 || cm > Sj) Sj = cm;
           }
-          Sx[j] = S;
+          Sx[j] = Sj;
           inv[j] = inv_j;
-          kx[j] = static_cast<unsigned char>(0x80 | k);
-        }
-      }
-      __syncthreads();
-      double v = INFINITY;
-      int vi = 0x7fffffff;
-      for (int c = tid; c < n_cand; c += T) {
-        const int j = list[c];
-        if (Sx[j] < v || (Sx[j] == v && j < vi)) {
-          v = Sx[j];
-          vi = j;
+          kx[j] = static_cast<unsigned char>((has_inv ? kHasInv : 0) | k);
+          if (Sj < v || (Sj == v && j < vi)) {
+            v = Sj;
+            vi = j;
+          }
         }
       }
       double rv;
       block_argmin(v, vi, red_v, red_i, rv, r);
-      if (r >= N) r = n_cand > 0 ? list[0] : 0;  // no finite value at all
+      if (r >= N) r = dense ? first_left(kx, N) : list[0];  // no finite value at all
+      // rows that lie closer together than the screening can tell apart will do so for the next picks too
+      dense = dense || 2 * n_cand > N - k;
     }
-    if (tid == 0) picks[k] = r;
+    if (tid == 0) {
+      picks[k] = r;
+      kx[r] |= kPicked;
+    }
   }
   __syncthreads();
 
@@ -624,15 +697,17 @@ cudaError_t launch_fps_dr(const Shape& s, const __nv_bfloat16* q_init, int N, fl
   return cudaGetLastError();
 }
 
-// Four warps up to 256 rows, with two or four tiles each (eight warps of two tiles: 233 us instead of 227
-// on the shape above: what a pick costs a warp besides its tiles is paid twice); up to 4096 rows eight
-// tiles per warp.  Rows that do
-// not fit in shared memory are read from global memory (L2) in every pass.
+// Four warps up to 256 rows, with two or four tiles each (eight warps of two tiles: 233 us instead of 227 on
+// 4608 instances of 256 rows of 128, call and state read: what a pick costs a warp besides its tiles is paid
+// twice); eight of four tiles up to 512 rows, two CTAs per SM where sixteen warps left room for one (1152
+// instances: 272 rows 154 -> 98 us, 512 rows 213 -> 175); above, up to 4096 rows, eight tiles per warp.  Rows
+// that do not fit in shared memory are read from global memory (L2) in every pass.
 template <int D>
 cudaError_t launch_fps_d(const Shape& s, const __nv_bfloat16* q_init, int N, float* cent, double* sums,
                          long long* counts, cudaStream_t st) {
   if (N <= 128) return launch_fps_dr<D, 4, 2, true>(s, q_init, N, cent, sums, counts, st);
   if (N <= 256) return launch_fps_dr<D, 4, 4, true>(s, q_init, N, cent, sums, counts, st);
+  if (N <= 512) return launch_fps_dr<D, 8, 4, true>(s, q_init, N, cent, sums, counts, st);
   if (N <= 2048 && fps_layout(N, D, 512, true).total <= kFpsResident)
     return launch_fps_dr<D, 16, 8, true>(s, q_init, N, cent, sums, counts, st);
   if (N <= 2048) return launch_fps_dr<D, 16, 8, false>(s, q_init, N, cent, sums, counts, st);
