@@ -23,6 +23,7 @@
 
 #include "bkv_device.cuh"
 #include "bkv_internal.h"
+#include "sincos.cuh"
 
 namespace bkv {
 namespace {
@@ -128,23 +129,24 @@ struct RopeChunk {
   long long pos[N];
 };
 
-// Rotary tables (and causal gaps) of a chunk of batch rows: block = one position, thread = one frequency
-// pair.  The angle is the fp64 product of position and frequency, its cosine and sine are CUDA's fp64
-// ones (within 2 ulp, far below what the fp64 -> fp32 -> bf16 rounding of a rotated query can see).
-// Formed on the host (576 pow, cos and sin for 8 recent slots and d = 128) the table cost a compress about
-// 50 us of host time before its first launch, and a copy kernel reading pinned memory.
+// Rotary tables (and causal gaps) of a chunk of batch rows: block = one position and 32 frequency pairs, one
+// thread each.  The angle is the fp64 product of position and frequency; its cosine and sine are within 0.501 ulp,
+// in integer arithmetic (in fp64 as accurate they took 4 us more).  Formed on the host (576 pow, cos and sin for 8 recent slots and d =
+// 128) the table cost a compress about 50 us of host time before its first launch, and a copy kernel reading
+// pinned memory; this kernel takes 6 us.
 template <int N>
-__global__ void __launch_bounds__(64) rope_table_kernel(const __grid_constant__ RopeChunk<N> c, int first_row, int W,
+__global__ void __launch_bounds__(32) rope_table_kernel(const __grid_constant__ RopeChunk<N> c, int first_row, int W,
                                                         int h, int rotate, double2* table, size_t row_stride, int* gaps,
                                                         int gap_max) {
-  const int row = blockIdx.x / (W + 1), slot = blockIdx.x % (W + 1), i = threadIdx.x;
+  const int at = blockIdx.x / (h / 32), i = (blockIdx.x % (h / 32)) * 32 + threadIdx.x;
+  const int row = at / (W + 1), slot = at % (W + 1);
+  const long long pos = c.pos[at];
+  double sn = 0.0, cs = 0.0;
+  if (rotate) sincos_accurate(__dmul_rn(static_cast<double>(pos), c.inv_freq[i]), sn, cs);
   grid_dependency_wait();  // an earlier compress may still read the table
-  const long long pos = c.pos[blockIdx.x];
   if (rotate) {
     double2* tab = table + static_cast<size_t>(first_row + row) * row_stride;
     float2* tab32 = reinterpret_cast<float2*>(tab + static_cast<size_t>(W + 1) * h);
-    double sn, cs;
-    sincos(__dmul_rn(static_cast<double>(pos), c.inv_freq[i]), &sn, &cs);
     tab[slot * h + i] = make_double2(cs, sn);
     tab32[slot * h + i] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
   }
@@ -169,8 +171,8 @@ cudaError_t launch_rope_chunks(int W, int h, int rows, const double* inv_freq, c
       for (int w = 0; w < W; ++w) pos[w] = recent_pos[static_cast<size_t>(r0 + r) * W + w];
       pos[W] = t_pos[r0 + r];
     }
-    const cudaError_t e = launch_dependent(rope_table_kernel<N>, static_cast<unsigned>(n * (W + 1)), static_cast<unsigned>(h),
-                                           0, st, c, r0, W, h, rotate, table, row_stride, gaps, gap_max);
+    const cudaError_t e = launch_dependent(rope_table_kernel<N>, static_cast<unsigned>(n * (W + 1) * (h / 32)), 32, 0, st, c,
+                                           r0, W, h, rotate, table, row_stride, gaps, gap_max);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
