@@ -491,7 +491,7 @@ def step_bench(args, wl, job, cfps: bool, steps: int, warmup: int, with_e2e: boo
                            "note": "per step: update (n_new queries per head) + beacon FPS + post-eviction merge"}
     kernels.update(kernel_table(prof, alg_bytes, prof_steps, hbm_gbs))
     ms, n = prof.get("rope_stage", (0.0, 0))
-    if n:  # the rotary table of a compress, 24 (W + 1) d / 2 bytes copied from pinned host memory
+    if n:  # the rotary table of a compress, computed on the device (the name is the profile's)
         kernels["rope_stage"] = {"ms_per_launch": ms / n, "launches": n}
     dom = max((k for k in kernels if "alg_bytes_per_launch" in kernels[k]),
               key=lambda k: kernels[k]["ms_per_launch"] * kernels[k]["launches"])

@@ -35,9 +35,10 @@
  * Streams.  All work is enqueued on the CUDA stream given to bkv_create (or
  * bkv_set_stream); calls return before it completes.  Outputs are valid once
  * that stream has been synchronised (bkv_sync does so and reports device-side
- * errors).  A compress passes its positions in kernel parameters and computes
- * its rotary table on the device: no call copies from host memory or waits for
- * the stream.  One context must not be used from two host threads at once.
+ * errors).  bkv_compress and bkv_compress_ragged pass their positions in kernel
+ * parameters and compute the rotary table on the device: they neither copy from
+ * host memory nor wait for the stream.  One context must not be used from two
+ * host threads at once.
  *
  * Errors.  Every call returns BKV_OK (0) or a negative code; nothing throws.
  * Argument errors are detected on the host before any work is enqueued and

@@ -26,8 +26,9 @@
 // beacons), exact: an element x with |x| < 2^E (E chosen per instance) goes
 // whole into one of two operands, the tile itself (|x| >= 2^(E-10), a multiple
 // of 2^(E-17)) or a second tile (smaller ones, multiples of 2^(E-27) for
-// |x| >= 2^(E-20)), whose sums over 128 rows stay below 2^24 grid steps, so the
-// fp32 accumulator never rounds.  The two sums of a (column, beacon) cell are
+// |x| >= 2^(E-20)), whose sums over 128 rows stay below 2^24 grid steps, so no
+// addition needs rounding (that the tensor cores then add without loss is not
+// documented: the tests hold it, with sums up to the limit).  The two sums of a (column, beacon) cell are
 // integers, added up over the tiles in two registers.  Elements outside
 // [2^(E-20), 2^E) (one in fifteen tiles of data of one scale has some) are zeroed in
 // the operands and added one by one, from a list in shared memory (past its end
@@ -941,7 +942,6 @@ __global__ void __launch_bounds__(kUThreads, 1)
   } else {
     // ---------------------------------------------------------------- builders: the unit-centroid operand
     const int wk = warp - kBuildWarp0;  // 0 .. 3
-    constexpr int kBatch = 1;
     for (int i = 0; i < n_my; ++i) {
       const int e = blockIdx.x + i * gridDim.x, pb = i & 1, slot = i & (kSlots - 1);
       if (wk == 0 && lane == 0 && i + 1 < n_my)
@@ -954,41 +954,34 @@ __global__ void __launch_bounds__(kUThreads, 1)
       uint32_t cmax = 0u;
       bool extreme = false;
 #pragma unroll 1
-      for (int b0 = wk; b0 < nbp; b0 += 4 * kBatch) {
-        float c[kBatch][D / 32];
+      for (int b = wk; b < nbp; b += 4) {
+        float c[D / 32];
 #pragma unroll
-        for (int u = 0; u < kBatch; ++u)
+        for (int k = 0; k < D / 32; ++k)
+          c[k] = b < nb ? a.cent[(static_cast<size_t>(e) * nb + b) * D + lane + 32 * k] : 0.f;
+        float n2 = 0.f;
 #pragma unroll
-          for (int k = 0; k < D / 32; ++k)
-            c[u][k] = b0 + 4 * u < nb ? a.cent[(static_cast<size_t>(e) * nb + b0 + 4 * u) * D + lane + 32 * k] : 0.f;
+        for (int k = 0; k < D / 32; ++k) n2 = fmaf(c[k], c[k], n2);
 #pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const int b = b0 + 4 * u;
-          if (b >= nbp) break;
-          float n2 = 0.f;
+        for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+        float big = 0.f;
 #pragma unroll
-          for (int k = 0; k < D / 32; ++k) n2 = fmaf(c[u][k], c[u][k], n2);
+        for (int k = 0; k < D / 32; ++k) big = fmaxf(big, fabsf(c[k]));
+        const bool ok = ((counted >> (b & 31)) & 1u) && b < nb && __any_sync(0xffffffffu, big != 0.f || n2 != n2);
+        if (ok) {
+          valid |= 1u << b;
+          cmax = max(cmax, __float_as_uint(big));
+          extreme |= !(n2 > 1e-30f && n2 < 1e30f);
+        }
+        const float inv = ok ? rsqrtf(n2) : 0.f;
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
-          float big = 0.f;
-#pragma unroll
-          for (int k = 0; k < D / 32; ++k) big = fmaxf(big, fabsf(c[u][k]));
-          const bool ok = ((counted >> (b & 31)) & 1u) && b < nb && __any_sync(0xffffffffu, big != 0.f || n2 != n2);
-          if (ok) {
-            valid |= 1u << b;
-            cmax = max(cmax, __float_as_uint(big));
-            extreme |= !(n2 > 1e-30f && n2 < 1e30f);
-          }
-          const float inv = ok ? rsqrtf(n2) : 0.f;
-#pragma unroll
-          for (int k = 0; k < D / 32; ++k) {
-            const int col = lane + 32 * k;
-            const float x = c[u][k] * inv;
-            const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-            const __nv_bfloat16 lo = __float2bfloat16_rn(x - __bfloat162float(hi));
-            *reinterpret_cast<__nv_bfloat16*>(bm + sw128_offset(b, col, bbox)) = hi;
-            *reinterpret_cast<__nv_bfloat16*>(bm + sw128_offset(nbp + b, col, bbox)) = lo;
-          }
+        for (int k = 0; k < D / 32; ++k) {
+          const int col = lane + 32 * k;
+          const float x = c[k] * inv;
+          const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+          const __nv_bfloat16 lo = __float2bfloat16_rn(x - __bfloat162float(hi));
+          *reinterpret_cast<__nv_bfloat16*>(bm + sw128_offset(b, col, bbox)) = hi;
+          *reinterpret_cast<__nv_bfloat16*>(bm + sw128_offset(nbp + b, col, bbox)) = lo;
         }
       }
       cmax = __reduce_max_sync(0xffffffffu, cmax);

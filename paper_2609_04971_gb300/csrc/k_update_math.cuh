@@ -1,8 +1,10 @@
 // Arithmetic shared by the beacon-update kernels (k_update.cu for many queries
-// per instance, k_update_small.cu for a few): double-float operations, the
-// exact per-column sums of bf16 values, the norm data of a centroid and the
-// exact re-decision of a close assignment.  Both kernels take their decisions
-// and sums with these same operations.
+// per instance, k_update_small.cu for a few, k_update_seq.cu for a run of decode
+// steps) and the seeding: double-float operations, norm data of centroids, the
+// exact re-decision of a close assignment, and the fold of a call's exact sum
+// into the running state.  The decisions of all of them are the same; the exact
+// sums of bf16 values in three fp32 parts serve the few-query kernels (the
+// batched kernel forms its sums on the tensor cores).
 #pragma once
 #include "bkv_device.cuh"
 

@@ -3,9 +3,9 @@
 // generated tokens (Algorithm 2's decode branch), G * n_new <= 32 per instance.
 //
 // One warp per instance, no tensor cores: at a handful of rows an instance is
-// too small for the batched kernel's pipeline (TMA ring, MMA screening,
-// accumulator and bookkeeping warps), whose per-instance handoffs then bound
-// the call.  The warp stages the call's queries in shared memory as fp32 and
+// too small for the batched kernel's pipeline (TMA ring, screening and one-hot
+// sums on the tensor cores, warps that take them out), whose per-instance
+// handoffs then bound the call.  The warp stages the call's queries in shared memory as fp32 and
 // gives each centroid row R = 32 / nb lanes (nb rounded up to a power of two):
 //   screening: the R lanes of beacon b stream its row from HBM once, in
 //     interleaved 16-byte chunks (adjacent lanes read adjacent chunks), and
@@ -24,8 +24,8 @@
 //     2e-4 |q| of the best enter the exact comparison: the screening error is
 //     far below 5e-5 |q|, so the exact maximum (and any exact tie with it)
 //     lies among them;
-//   sums: per touched beacon, the rows assigned to it are added as the same
-//     three exact fp32 parts, turned into round(sum * 2^40), added once to the
+//   sums: per touched beacon, the rows assigned to it are added as three
+//     exact fp32 parts (k_update_math.cuh), turned into round(sum * 2^40), added once to the
 //     fp64 running sum (fold_sum: exact integer addition and one rounding, no
 //     fp64 arithmetic in the common case), and c = fp32(sum / count) to within
 //     one ulp from double-float arithmetic, as in the batched kernel's fold.  The running
